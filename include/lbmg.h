@@ -117,7 +117,9 @@ typedef struct lbmg_stats {
     double initial_residual[4];
     float ms_total;          /* device time of the solve, CUDA events */
     float ms_fine_smooth;    /* device time of the finest-level smoothing sweeps summed over all cycles
-                                (events in the per-cycle graph; %globaltimer in the persistent solve) */
+                                (events in the per-cycle graph; %globaltimer in the persistent solve);
+                                where the finest level's sweeps are tiled it includes the residual and
+                                the prolongation, which their launches do */
     int learned;             /* 1 if the learned correction preceded the cycles (lbmg_learned_enable) */
     int learned_fallback;    /* 1 if an iteration with it raised a residual and the solve went on with
                                 plain cycles (the acceptance test) */
@@ -326,7 +328,10 @@ int lbmg_launch_counts(lbmg_handle h, int precision, int *assemble, int *project
  * least 2% faster).  Threads per row 8 and 16 read the matrix in CSR order; 4 reads
  * a packed copy in which groups of 8 rows of one colour with equal quad counts
  * ceil(len / 4) store their entries quad-interleaved, so that each warp load is 256
- * aligned contiguous bytes.  Results are also kept in a process-wide cache
+ * aligned contiguous bytes.  Levels of up to some ten thousand rows also have the tiled
+ * sweep: blocks walk all colours of a sweep on a tile of rows and its rim in shared
+ * memory, one or two launches per sweep instead of eight; it is the default there, and
+ * the tuner keeps it unless a shape is faster.  Results are also kept in a process-wide cache
  * keyed by (device name, precision, kernel, lanes, rows, non-zeros): levels of
  * any handle that match an entry are not timed again.  The levels' cycle work
  * vectors are overwritten; they carry no state between calls.  Captured cycle
@@ -336,7 +341,8 @@ int lbmg_launch_counts(lbmg_handle h, int precision, int *assemble, int *project
  */
 int lbmg_autotune(lbmg_handle h, int nrhs, int precision, int reps, int *timed, void *stream);
 /* launch shapes of level d for `precision`: out[4] = Gauss-Seidel sweep (threads per row,
-   threads per block), residual (threads per row, threads per block).  Host only. */
+   threads per block), residual (threads per row, threads per block).  Host only.  (A level
+   whose sweeps are tiled has the default shape.) */
 int lbmg_launch_shape(lbmg_handle h, int d, int precision, int *out);
 /* device time (ms) that the last lbmg_autotune measured on this handle for level d's chosen
    shapes: ms[0] one Gauss-Seidel sweep (8 chained colour launches), ms[1] one residual
@@ -348,13 +354,14 @@ int lbmg_tuned_times(lbmg_handle h, int d, int precision, float *ms);
    sweeps of one smoothing) in one cooperative launch of the packed-copy kernel, whose
    blocks meet at a bounded grid barrier between colours (a timeout gives
    LBMG_DEVICE_TIMEOUT); it computes exactly what the colour launches of tpr = 4 compute.
-   LBMG_INVALID_ARG otherwise.  Results change only by the summation order inside a row.
-   Host only. */
+   LBMG_INVALID_ARG otherwise.  A sweep shape set by hand turns the level's tiled sweep off.
+   Results change only by the summation order inside a row.  Host only. */
 int lbmg_set_launch_shape(lbmg_handle h, int d, int precision, int kind, int tpr, int tpb);
 /* options.host_check of an existing handle (0 or 1; LBMG_INVALID_ARG otherwise).  Host only. */
 int lbmg_set_host_check(lbmg_handle h, int on);
 /* write / read the process-wide tuning cache as text, one entry per line:
-   device fp64 kind lanes rows nnz threads_per_row threads_per_block.
+   device fp64 kind lanes rows nnz threads_per_row threads_per_block [grid], the last the
+   whole-sweep kernel's blocks, or -1 for the tiled sweep.
    Load merges valid lines and returns LBMG_INVALID_ARG if the file cannot be
    opened or a line is malformed (valid lines are still taken). */
 int lbmg_tune_cache_save(const char *path);

@@ -13,8 +13,8 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "liblbmg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU = ["assemble.cu", "relax.cu", "packed.cu", "persist.cu", "narrow.cu", "learned.cu", "noalloc.cu", "cmcf.cu", "lobpcg.cu", "tune.cu", "clip.cu", "basis.cu", "api.cu"]
-CPP = ["hier.cpp", "batch.cpp"]
+CU = ["assemble.cu", "relax.cu", "packed.cu", "tile.cu", "persist.cu", "narrow.cu", "learned.cu", "noalloc.cu", "cmcf.cu", "lobpcg.cu", "tune.cu", "clip.cu", "basis.cu", "api.cu"]
+CPP = ["hier.cpp", "batch.cpp", "tile_plan.cpp"]
 
 
 def _nvcc():
@@ -26,7 +26,7 @@ def _nvcc():
 
 def sources():
     return [os.path.join(CSRC, f) for f in CU + CPP] + [
-        os.path.join(CSRC, h) for h in ("hier.h", "lbmg_internal.h")] + [
+        os.path.join(CSRC, h) for h in ("hier.h", "tile_plan.h", "lbmg_internal.h")] + [
         os.path.join(os.path.dirname(HERE), "include", "lbmg.h")]
 
 

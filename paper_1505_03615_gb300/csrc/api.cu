@@ -54,6 +54,13 @@ bool on_device(const void *p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// the live right-hand sides of a call, for the kernels that leave out the padding of three to four
+struct LiveLanes {
+    Ctx &c;
+    LiveLanes(Ctx &ctx, int n) : c(ctx) { c.lanes = n; }
+    ~LiveLanes() { c.lanes = 0; }
+};
+
 inline int stride_for(int nrhs) { return nrhs == 1 ? 1 : (nrhs == 2 ? 2 : 4); }
 
 __global__ void to_double_kernel(const float *__restrict__ a, double *__restrict__ b, int64_t n) {
@@ -225,6 +232,7 @@ template <> struct P<float> {
     static float *x(DevLevel &L) { return L.x32; }
     static float *b(DevLevel &L) { return L.b32; }
     static float *r(DevLevel &L) { return L.r32; }
+    static float *y(DevLevel &L) { return L.y32; }
     static const float *A(DevLevel &L) { return L.A32; }
     static const float *dinv(DevLevel &L) { return L.dinv32; }
     static const float *inv(Ctx &c) { return c.cinv32; }
@@ -233,14 +241,30 @@ template <> struct P<double> {
     static double *x(DevLevel &L) { return L.x64; }
     static double *b(DevLevel &L) { return L.b64; }
     static double *r(DevLevel &L) { return L.r64; }
+    static double *y(DevLevel &L) { return L.y64; }
     static const double *A(DevLevel &L) { return L.A64; }
     static const double *dinv(DevLevel &L) { return L.dinv64; }
     static const double *inv(Ctx &c) { return c.cinv64; }
 };
 
+// whether the level's sweeps run in the tiled kernel: it has a plan and no other launch shape was chosen
+template <class T>
+bool tiled(const Ctx &c, const DevLevel &L) {
+    return c.smoother == LBMG_GS_COLOURED && L.tparts > 0 && L.shape[sizeof(T) == 8][kShapeSmooth].tile;
+}
+
 template <class T>
 void enqueue_smooth(Ctx &c, DevLevel &L, int R, int sweeps, bool forward, cudaStream_t s, Chain *ch, int skip = 0) {
-    if (c.smoother == LBMG_JACOBI) {
+    if (tiled<T>(c, L)) {
+        // from one vector to the other and back; the rows behind ns keep their place in x
+        TileVec<T> v{P<T>::x(L), P<T>::y(L)};
+        for (int sw = 0; sw < sweeps; sw++)
+            launch_tile_sweep<T>(c, L, forward, v, P<T>::b(L), (T *)nullptr, R, s, ch);
+        if (v.cur) {
+            cudaMemcpyAsync(v.x, v.y, (size_t)L.ns * R * sizeof(T), cudaMemcpyDeviceToDevice, s);
+            if (ch) ch->cut();
+        }
+    } else if (c.smoother == LBMG_JACOBI) {
         for (int sw = 0; sw < sweeps; sw++) {
             launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch);
             launch_jacobi_update<T>(L, P<T>::dinv(L), P<T>::r(L), P<T>::x(L), (T)c.omega, R, s);
@@ -264,8 +288,11 @@ inline void record(cudaEvent_t e, cudaStream_t s, Chain *ch) {
 // Every coarser correction is zeroed by the restriction that fills its right-hand
 // side, so the kernels of the cycle follow one another with no memset between
 // them and run as one chain of dependent launches.
+// Tiled levels take a launch or two per sweep, the residual with the last sweep down, the prolongation in
+// the first one up (timed: the events bracket these too).
+// zero: e is zero on entry (the tiled finest level does not read it then).
 template <class T>
-void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int top = -1) {
+void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int top = -1, bool zero_start = true) {
     if (top < 0) top = c.D;
     // bottom levels: from shared memory in one block (FP32), from global memory in
     // one block (levels of at most narrow_max rows), or one launch per phase down to d0
@@ -277,15 +304,34 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
         else if (std::min(c.persist_dn, top) >= c.d0) { bottom = kL2; dn = std::min(c.persist_dn, top); }
     }
     int skip = 0;   // colour steps of the next level's first sweep that its restriction did
+    TileVec<T> vec[kMaxDepth + 1];
+    auto tile = [&](int d) { return c.nu1 > 0 && c.nu2 > 0 && tiled<T>(c, c.lev[d]); };
     for (int d = top; d > dn; d--) {
         DevLevel &L = c.lev[d], &Lc = c.lev[d - 1];
         launch_coarse_apply<T>(c, L, P<T>::inv(c), P<T>::b(L), P<T>::x(L), R, s, ch);
         if (timed && d == top) record(c.ev_smooth[0], s, ch);
-        enqueue_smooth<T>(c, L, R, c.nu1, true, s, ch, skip);
-        if (timed && d == top) record(c.ev_smooth[1], s, ch);
-        launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch);
+        if (tile(d)) {
+            // each of the nu1 + nu2 sweeps moves the vector to the other buffer; the last has to write x
+            TileVec<T> &v = vec[d];
+            v = TileVec<T>{P<T>::x(L), P<T>::y(L)};
+            const unsigned all = (1u << L.tparts) - 1u;
+            v.cur = (c.nu1 + c.nu2) & 1 ? all : 0u;
+            if (d != top || zero_start) v.zero = all;
+            else if (v.cur) {
+                cudaMemcpyAsync(v.y, v.x, (size_t)L.ns * R * sizeof(T), cudaMemcpyDeviceToDevice, s);
+                ch->cut();
+            }
+            for (int q = 0; q < c.nu1; q++)
+                launch_tile_sweep<T>(c, L, true, v, P<T>::b(L), q + 1 == c.nu1 ? P<T>::r(L) : (T *)nullptr, R, s, ch);
+            if (timed && d == top) record(c.ev_smooth[1], s, ch);
+        } else {
+            enqueue_smooth<T>(c, L, R, c.nu1, true, s, ch, skip);
+            if (timed && d == top) record(c.ev_smooth[1], s, ch);
+            launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch);
+        }
         // the shared-memory bottom starts level dn from zero itself; the dense solve overwrites d0
-        const bool zero = bottom == kSmem ? d - 1 > dn : (bottom == kL2 || d - 1 > c.d0);
+        // (and a tiled level's first sweep starts from zero without reading it)
+        const bool zero = (bottom == kSmem ? d - 1 > dn : (bottom == kL2 || d - 1 > c.d0)) && !(d - 1 > dn && tile(d - 1));
         // a level that this loop smooths next (Gauss-Seidel, from zero) gets its first colour step
         // from the restriction that zeroes it
         const bool fuse = zero && d - 1 > dn && c.smoother != LBMG_JACOBI && c.nu1 > 0;
@@ -300,6 +346,16 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
     }
     for (int d = dn + 1; d <= top; d++) {
         DevLevel &L = c.lev[d];
+        if (tile(d)) {
+            TileVec<T> &v = vec[d];
+            v.xc = P<T>::x(c.lev[d - 1]);
+            v.prolong = (1u << L.tparts) - 1u;
+            if (timed && d == top) record(c.ev_smooth[2], s, ch);
+            for (int q = 0; q < c.nu2; q++)
+                launch_tile_sweep<T>(c, L, false, v, P<T>::b(L), (T *)nullptr, R, s, ch);
+            if (timed && d == top) record(c.ev_smooth[3], s, ch);
+            continue;
+        }
         launch_prolong_add<T>(L, P<T>::x(c.lev[d - 1]), P<T>::x(L), R, s, ch);
         if (timed && d == top) record(c.ev_smooth[2], s, ch);
         enqueue_smooth<T>(c, L, R, c.nu2, false, s, ch);
@@ -340,8 +396,8 @@ void enqueue_cycle_level(Ctx &c, int d, int R, cudaStream_t s, Chain *ch) {
 
 // one cycle on A e = b at the finest level, e zero on entry
 template <class T>
-void enqueue_cycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch) {
-    if (c.gamma == 1 && !c.coarse_smooth) enqueue_vcycle<T>(c, R, s, timed, ch);
+void enqueue_cycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, bool zero_start = true) {
+    if (c.gamma == 1 && !c.coarse_smooth) enqueue_vcycle<T>(c, R, s, timed, ch, -1, zero_start);
     else enqueue_cycle_level<T>(c, c.D, R, s, ch);
 }
 
@@ -370,7 +426,7 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
     if (precision == LBMG_MIXED) {
         if (c.learned_on) learned_enqueue(c, R, precision, s, &ch);   // the cycle starts from the correction
         else launch_to_float(c.rs, F.b32, m, s, F.x32, &ch);
-        enqueue_cycle<float>(c, R, s, timed, &ch);
+        enqueue_cycle<float>(c, R, s, timed, &ch, !c.learned_on);
         // x += e, and the outer residual with FP64 values carried as FP32 pairs (GB300's FP64
         // rate would bound an FP64 residual of the finest level)
         if (pair_iterate(c, precision, false)) {
@@ -387,7 +443,7 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
             cudaMemcpyAsync(F.b64, c.rs, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
             cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
         }
-        enqueue_cycle<double>(c, R, s, timed, &ch);
+        enqueue_cycle<double>(c, R, s, timed, &ch, !c.learned_on);
         launch_add_double(c.xs, F.x64, m, s);
         ch.cut();
     }
@@ -465,7 +521,7 @@ int get_graph(lbmg_handle h, int R, int precision, bool pcg, cudaGraphExec_t *ou
     Ctx &c = h->c;
     GraphCache &g = c.graph;
     if (g.exec && g.R == R && g.precision == precision && g.nu1 == c.nu1 && g.nu2 == c.nu2 && g.smoother == c.smoother &&
-        g.pcg == (int)pcg && g.cond == 0 && g.learned == c.learned_on) {
+        g.pcg == (int)pcg && g.cond == 0 && g.learned == c.learned_on && g.lanes == c.lanes) {
         *out = g.exec;
         return LBMG_OK;
     }
@@ -486,6 +542,7 @@ int get_graph(lbmg_handle h, int R, int precision, bool pcg, cudaGraphExec_t *ou
     g.R = R; g.precision = precision; g.nu1 = c.nu1; g.nu2 = c.nu2; g.smoother = c.smoother; g.pcg = pcg;
     g.cond = 0;
     g.learned = c.learned_on;
+    g.lanes = c.lanes;
     *out = g.exec;
     return LBMG_OK;
 }
@@ -548,7 +605,7 @@ int get_cond_graph(lbmg_handle h, int R, int precision, bool pcg, cudaGraphExec_
     Ctx &c = h->c;
     GraphCache &g = c.graph;
     if (g.exec && g.R == R && g.precision == precision && g.nu1 == c.nu1 && g.nu2 == c.nu2 && g.smoother == c.smoother &&
-        g.pcg == (int)pcg && g.cond == 1 && g.learned == c.learned_on) {
+        g.pcg == (int)pcg && g.cond == 1 && g.learned == c.learned_on && g.lanes == c.lanes) {
         *out = g.exec;
         return LBMG_OK;
     }
@@ -563,6 +620,7 @@ int get_cond_graph(lbmg_handle h, int R, int precision, bool pcg, cudaGraphExec_
     g.R = R; g.precision = precision; g.nu1 = c.nu1; g.nu2 = c.nu2; g.smoother = c.smoother; g.pcg = pcg;
     g.cond = 1;
     g.learned = c.learned_on;
+    g.lanes = c.lanes;
     *out = g.exec;
     return LBMG_OK;
 }
@@ -586,6 +644,81 @@ int read_norms(lbmg_handle h, int R, cudaStream_t s, double *out4) {
 int check_level(lbmg_handle h, int d) {
     if (!h) return LBMG_INVALID_ARG;
     if (d < h->c.d0 || d > h->c.D) return LBMG_INVALID_ARG;
+    return LBMG_OK;
+}
+
+// Tile plans of a level's sweeps (tile.cu).  A level whose tiles would not fit keeps the colour launches.
+int build_tiles(lbmg_handle h, const HostLevel &hl, DevLevel &L, int sms) {
+    if (L.ns > kTileLevel32) return LBMG_OK;
+    L.shape[1][kShapeSmooth].tile = L.ns <= kTileLevel64;
+    int parts = 1, nt = 1;
+    tile_shape(L.ns, sms, &parts, &nt);
+    const int per = 8 / parts;
+    const bool fused = parts == 1;
+    int down[8], up[8];
+    for (int q = 0; q < 8; q++) { down[q] = q; up[q] = 7 - q; }
+    TileCut cut;
+    cut_tiles(hl, nt, cut);
+    TilePlan plan;
+    if (nt > 1) {
+        // even out what the tiles process, then halve those whose rim is far above the others'
+        if (!build_tile_plan(hl, cut, down, per, fused, plan)) return LBMG_OK;
+        rebalance_tiles(plan, cut);
+        for (int k = 0; k < 3 && nt > sms; k++) {
+            if (!build_tile_plan(hl, cut, down, per, fused, plan)) return LBMG_OK;
+            int64_t sum = 0;
+            for (int t = 0; t < plan.ntile; t++) sum += plan.info[(size_t)t * kTileInfo];
+            if (!split_tiles(plan, (int)(1.4 * sum / plan.ntile) + 64, cut)) break;
+        }
+    }
+    struct Job { TileDev *t; const int *seq; int nsteps; bool residual; };
+    std::vector<Job> jobs;
+    for (int p = 0; p < parts; p++) {
+        jobs.push_back({&L.tile[0][p], down + per * p, per, fused});
+        jobs.push_back({&L.tile[1][p], up + per * (parts - 1 - p), per, false});
+    }
+    if (!fused) jobs.push_back({&L.tres, down, 0, true});
+    for (const Job &j : jobs) {
+        TileDev &t = *j.t;
+        if (!build_tile_plan(hl, cut, j.seq, j.nsteps, j.residual, plan) || !tile_fits(plan, t)) return LBMG_OK;
+        std::vector<int64_t> gquad((size_t)plan.groups);
+        for (int q = 0; q < plan.ntile; q++) {
+            const int32_t *f = &plan.info[(size_t)q * kTileInfo], *cum = &plan.cum[(size_t)q * (plan.maxgrp + 1)];
+            for (int g = 0; g < f[5 + plan.nsteps]; g++) gquad[(size_t)f[3] + g] = f[4] + (int64_t)cum[g];
+        }
+        std::vector<int32_t> loc((size_t)plan.ntile * t.maxloc, 0);
+        for (int q = 0; q < plan.ntile; q++)
+            for (int i = 0; i < plan.info[(size_t)q * kTileInfo]; i++)
+                loc[(size_t)q * t.maxloc + i] = plan.loc[(size_t)q * plan.maxloc + i];
+        LBMG_TRY(h->upload(&t.info, plan.info));
+        LBMG_TRY(h->upload(&t.loc, loc));
+        std::vector<int32_t> tcum((size_t)plan.ntile * t.maxgrp, 0);
+        for (int q = 0; q < plan.ntile; q++)
+            std::copy_n(plan.cum.begin() + (size_t)q * (plan.maxgrp + 1), plan.maxgrp + 1, tcum.begin() + (size_t)q * t.maxgrp);
+        LBMG_TRY(h->upload(&t.cum, tcum));
+        LBMG_TRY(h->upload(&t.map, plan.map));
+        LBMG_TRY(h->upload(&t.row, plan.row));
+        LBMG_TRY(h->upload(&t.qgroup, plan.qgroup));
+        LBMG_TRY(h->upload(&t.gquad, gquad));
+        LBMG_TRY(h->alloc(&t.s32, tile_stream_bytes(t, false)));
+        LBMG_TRY(h->alloc(&t.s64, tile_stream_bytes(t, true)));
+        uint16_t *col = nullptr, *slot = nullptr;   // only until the streams hold them
+        cudaError_t e = cudaMalloc((void **)&col, std::max<size_t>(plan.col.size(), 1) * 2);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&slot, std::max<size_t>(plan.slot.size(), 1) * 2);
+        if (e == cudaSuccess && !plan.col.empty())
+            e = cudaMemcpy(col, plan.col.data(), plan.col.size() * 2, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && !plan.slot.empty())
+            e = cudaMemcpy(slot, plan.slot.data(), plan.slot.size() * 2, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = launch_tile_layout(t, col, slot, nullptr);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+        cudaFree(col);
+        cudaFree(slot);
+        LBMG_CK(e);
+    }
+    LBMG_TRY(h->alloc(&L.y64, 4 * (size_t)L.n));
+    LBMG_TRY(h->alloc(&L.y32, 4 * (size_t)L.n));
+    L.tparts = parts;
+    L.tfused = fused;
     return LBMG_OK;
 }
 
@@ -615,6 +748,10 @@ int upload_hierarchy(lbmg_handle h) {
     }
     c.ncblk = (int)(c.cblk_host.size() / 5);
     LBMG_TRY(h->upload(&c.cblk, c.cblk_host));
+    const bool tiles = tile_setup();
+    int dev = 0, sms = 0;
+    LBMG_CK(cudaGetDevice(&dev));
+    LBMG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     for (int d = c.d0; d <= c.D; d++) {
         HostLevel &hl = H.lev[d];
         DevLevel &L = c.lev[d];
@@ -672,6 +809,7 @@ int upload_hierarchy(lbmg_handle h) {
                 LBMG_TRY(h->alloc(&L.pk_v2, (size_t)L.pk_total));
             }
         }
+        if (d > c.d0 && L.ns > 0 && c.smoother == LBMG_GS_COLOURED && tiles) LBMG_TRY(build_tiles(h, hl, L, sms));
         const size_t v4 = 4 * (size_t)L.n;
         LBMG_TRY(h->alloc(&L.x64, v4));
         LBMG_TRY(h->alloc(&L.b64, v4));
@@ -1163,6 +1301,7 @@ int lbmg_assemble(lbmg_handle h, double t, void *stream) {
     for (int d = c.D - 1; d >= c.d0; d--) launch_galerkin(c, d, t, s);
     for (int d = c.d0; d <= c.D; d++) launch_inverse_diag(c.lev[d], c.diag_part, s);
     for (int d = c.d0 + 1; d <= c.D; d++) launch_packed_fill(c.lev[d], s);
+    for (int d = c.d0 + 1; d <= c.D; d++) launch_tile_fill(c.lev[d], s);
     cudaMemsetAsync(c.flag, 0, sizeof(int), s);
     launch_coarse_factor(c, h->lev_rp, h->lev_ci, h->lev_A, s);
     narrow_smem_refresh(c, s);
@@ -1368,6 +1507,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
     Ctx &c = h->c;
     cudaStream_t s = (cudaStream_t)stream;
     const int R = stride_for(nrhs);
+    const LiveLanes live(c, nrhs);
     DevLevel &Fl = c.lev[c.D];
     const size_t cnt = (size_t)Fl.n * nrhs;
     const double *rd, *xin;
@@ -1672,6 +1812,7 @@ int lbmg_smooth(lbmg_handle h, int d, const double *rhs, double *x, int nrhs, in
     cudaStream_t s = (cudaStream_t)stream;
     DevLevel &L = h->c.lev[d];
     const int R = stride_for(nrhs);
+    const LiveLanes live(h->c, nrhs);
     const size_t cnt = (size_t)L.n * nrhs;
     const int64_t m = (int64_t)L.n * R;
     const double *bd, *xd;
@@ -1751,6 +1892,11 @@ int lbmg_launch_counts(lbmg_handle h, int precision, int *assemble, int *project
         cyc = 1;   // the one-block bottom cycle, or the coarse apply
         for (int d = bottom + 1; d <= c.D; d++) {   // sweeps, residual, restriction, prolongation
             const DevLevel &L = c.lev[d];
+            if (c.nu1 > 0 && c.nu2 > 0 && c.smoother != LBMG_JACOBI && L.tparts > 0 &&
+                L.shape[precision == LBMG_FP64][kShapeSmooth].tile) {   // sweeps, residual, restriction
+                cyc += (c.nu1 + c.nu2) * L.tparts + (L.tfused ? 0 : 1) + 1 + (L.ncb > 0);
+                continue;
+            }
             const bool whole = precision == LBMG_MIXED && c.smoother != LBMG_JACOBI &&
                                L.shape[0][kShapeSmooth].tpb == kSweepShapeTpb && L.pk_map && c.sweep_bar;
             if (whole) cyc += (c.nu1 > 0) + (c.nu2 > 0);   // one cooperative launch per smoothing
@@ -1823,6 +1969,7 @@ int lbmg_set_launch_shape(lbmg_handle h, int d, int precision, int kind, int tpr
     LaunchShape &sh = h->c.lev[d].shape[precision == LBMG_FP64][kind];
     sh.tpr = tpr;
     sh.tpb = tpb;
+    sh.tile = false;
     h->c.lev[d].tuned_ms[precision == LBMG_FP64][kind] = 0.f;
     if (h->c.graph.exec) { cudaGraphExecDestroy(h->c.graph.exec); h->c.graph.exec = nullptr; }
     return LBMG_OK;

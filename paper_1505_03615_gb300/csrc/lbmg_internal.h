@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "hier.h"
+#include "tile_plan.h"
 
 namespace lbmg {
 
@@ -19,6 +20,7 @@ constexpr int kNormBlocks = 256;  // partial sums of the two-pass norm reduction
 struct LaunchShape {
     int tpr = 4, tpb = 256;   // Gauss-Seidel with tpb = 1024: the whole-sweep cooperative kernel (packed.cu)
     int grid = 0;             // its blocks (0: one per SM; fewer make the grid barrier cheaper on small levels)
+    bool tile = true;         // the tiled kernel (tile.cu) where the level has a plan; tpr, tpb are then unused
 };
 constexpr int kSweepShapeTpb = 1024;
 enum { kShapeSmooth = 0, kShapeResidual = 1 };
@@ -72,6 +74,16 @@ struct PkRuns {
     int g[kPkRuns] = {0}, b[kPkRuns] = {0}, q[kPkRuns] = {0};
 };
 
+// device copy of a tile plan (tile_plan.h): the streams hold slots, columns, inverse diagonals and values
+struct TileDev {
+    int ntile = 0, nsteps = 0, maxloc = 0, maxcomp = 0, maxgrp = 0, maxquads = 0;
+    int64_t groups = 0, quads = 0;
+    int ring[2][3] = {{0}};                // [FP64][R = 1, 2, 4] groups in flight per warp
+    int *info = nullptr, *loc = nullptr, *cum = nullptr, *map = nullptr, *row = nullptr, *qgroup = nullptr;
+    int64_t *gquad = nullptr;              // [groups] quads before each group
+    unsigned char *s32 = nullptr, *s64 = nullptr;
+};
+
 struct DevLevel {
     int d = 0, n = 0;
     int ns = 0;                            // rows [0, ns) are smoothed; [ns, n) belong to coarsest blocks
@@ -93,6 +105,12 @@ struct DevLevel {
     // V-cycle work vectors, room for [n][4]
     double *x64 = nullptr, *b64 = nullptr, *r64 = nullptr;
     float *x32 = nullptr, *b32 = nullptr, *r32 = nullptr;
+    double *y64 = nullptr;                 // the tiled sweep's other vector (it reads one, writes the other)
+    float *y32 = nullptr;
+    TileDev tile[2][kTileParts];           // sweeps 0..7 and 7..0, each in tparts launches of 8 / tparts colours;
+    int tparts = 0;                        // part q: colours from 8 q / tparts on (0: no plan)
+    bool tfused = false;                   // a sweep 0..7 can form the residual in its launch, else tres does
+    TileDev tres;
     // packed copy of A for the row kernels (packed.cu): per colour, 8-row groups of rows with
     // equal quad counts, entries quad-interleaved across the group; null pk_map when not built
     int2 *pk_gq = nullptr;                 // [ngroups] (base / 32, quads)
@@ -140,6 +158,7 @@ struct GraphCache {
     int R = 0, precision = -1, nu1 = -1, nu2 = -1, smoother = -1, pcg = -1;
     int cond = -1;   // 1: the whole solve (conditional WHILE node), 0: one iteration
     int learned = -1;   // the learned correction in front of each cycle
+    int lanes = -1;
 };
 
 // Device-side control of a solve that runs as one graph launch: a conditional WHILE node
@@ -225,6 +244,7 @@ struct Ctx {
     double *pin_io = nullptr;
     size_t pin_io_bytes = 0;
     bool assembled = false;
+    int lanes = 0;                // live right-hand sides of the running call (0: all R components)
     double t = 0;
     cudaStream_t capture_stream = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -336,6 +356,24 @@ void launch_add_pair(const float *e, float *xh, float *xl, int64_t n, cudaStream
 bool launch_packed_sweep(const DevLevel &L, const int *seq, int nseq, const float *dinv, const float *b, float *x,
                          int R, unsigned *bar, int *status, int blocks, cudaStream_t s);
 int packed_sweep_blocks(int R);   // the grid of the sweep kernel (resident blocks per SM x SMs)
+
+// ----- tiled sweep (tile.cu) -----
+bool tile_setup();
+bool tile_fits(const TilePlan &p, TileDev &t);   // sets t's sizes; false when a launch would not fit a block
+size_t tile_stream_bytes(const TileDev &t, bool fp64);
+cudaError_t launch_tile_layout(const TileDev &t, const uint16_t *col, const uint16_t *slot, cudaStream_t s);
+void launch_tile_fill(const DevLevel &L, cudaStream_t s);
+// The level's vector during tiled sweeps: part q of the rows is in y when bit q of cur is set, else in x
+// (each launch reads one and writes the other), zero where bit q of zero is set, and still lacks the
+// prolonged coarse correction xc where bit q of prolong is set.
+template <class T> struct TileVec {
+    T *x, *y;
+    unsigned cur = 0, zero = 0, prolong = 0;
+    const T *xc = nullptr;
+};
+// a sweep over the colours 0..7 (forward) or 7..0; r (forward only, may be null): the residual b - A x after it
+template <class T> void launch_tile_sweep(const Ctx &c, const DevLevel &L, bool forward, TileVec<T> &v, const T *b, T *r,
+                                          int R, cudaStream_t s, Chain *ch);
 
 // ----- kernels (relax.cu) -----
 // vectors below are [n][R] with stride R in {1, 2, 4} (3 right-hand sides padded to 4)

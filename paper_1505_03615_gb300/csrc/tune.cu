@@ -46,6 +46,7 @@ template <> struct V<float> {
     static float *x(DevLevel &L) { return L.x32; }
     static float *b(DevLevel &L) { return L.b32; }
     static float *r(DevLevel &L) { return L.r32; }
+    static float *y(DevLevel &L) { return L.y32; }
 };
 template <> struct V<double> {
     static const double *A(const DevLevel &L) { return L.A64; }
@@ -53,6 +54,7 @@ template <> struct V<double> {
     static double *x(DevLevel &L) { return L.x64; }
     static double *b(DevLevel &L) { return L.b64; }
     static double *r(DevLevel &L) { return L.r64; }
+    static double *y(DevLevel &L) { return L.y64; }
 };
 
 // device time of one sweep (8 colours) or one residual with the level's current shape
@@ -63,8 +65,11 @@ cudaError_t time_kernel(Ctx &c, DevLevel &L, int kind, int R, int reps, cudaEven
     if (e != cudaSuccess) return e;
     Chain ch;
     ch.on = c.pdl != 0;   // the capture stream is an ordinary stream
+    TileVec<T> tv{V<T>::x(L), V<T>::y(L)};
     for (int q = 0; q < reps; q++) {
-        if (kind == kShapeSmooth) {
+        if (kind == kShapeSmooth && L.tparts > 0 && L.shape[sizeof(T) == 8][kind].tile) {
+            launch_tile_sweep<T>(c, L, true, tv, V<T>::b(L), (T *)nullptr, R, cs, &ch);
+        } else if (kind == kShapeSmooth) {
             launch_sweeps<T>(c, L, 1, true, V<T>::A(L), V<T>::dinv(L), V<T>::b(L), V<T>::x(L), R, cs, &ch);
         } else {
             launch_residual<T>(L, V<T>::A(L), V<T>::b(L), V<T>::x(L), V<T>::r(L), R, cs, L.ns, &ch);
@@ -102,6 +107,7 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
         const size_t bytes = (size_t)L.n * 4 * sizeof(T);
         e = cudaMemsetAsync(V<T>::x(L), 0, bytes, c.capture_stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(V<T>::b(L), 0, bytes, c.capture_stream);
+        if (e == cudaSuccess && L.tparts > 0) e = cudaMemsetAsync(V<T>::y(L), 0, bytes, c.capture_stream);
         for (int kind = 0; kind < 2 && e == cudaSuccess; kind++) {
             const Key key{dev, fp64, kind, R, (int64_t)L.ns, L.nnz};
             {
@@ -114,6 +120,8 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
                 }
             }
             LaunchShape best = LaunchShape(), dflt = LaunchShape();
+            best.tile = dflt.tile = false;
+            const LaunchShape before = L.shape[fp64][kind];
             float best_ms = 0.f, dflt_ms = 0.f;
             bool have = false;
             for (int a = 0; a < 3 && e == cudaSuccess; a++)
@@ -121,6 +129,7 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
                     LaunchShape sh;
                     sh.tpr = kTpr[a];
                     sh.tpb = kTpb[b];
+                    sh.tile = false;
                     L.shape[fp64][kind] = sh;
                     float ms = 0.f;
                     e = time_kernel<T>(c, L, kind, R, reps, e0, e1, &ms);
@@ -128,7 +137,7 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
                     if (sh.tpr == dflt.tpr && sh.tpb == dflt.tpb) dflt_ms = ms;
                     if (!have || ms < best_ms) { best = sh; best_ms = ms; have = true; }
                 }
-            if (e != cudaSuccess) { L.shape[fp64][kind] = dflt; break; }
+            if (e != cudaSuccess) { L.shape[fp64][kind] = before; break; }
             // keep the default unless another shape is clearly faster (timing noise)
             if (dflt_ms > 0.f && best_ms > 0.98f * dflt_ms) { best = dflt; best_ms = dflt_ms; }
             // FP32 sweeps of a level with a packed copy: the whole-sweep cooperative kernel, kept when it
@@ -140,6 +149,7 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
                     LaunchShape sw;
                     sw.tpr = 4;
                     sw.tpb = kSweepShapeTpb;
+                    sw.tile = false;
                     sw.grid = div == 1 ? 0 : std::max(1, c.sweep_blocks[R] / div);
                     L.shape[fp64][kind] = sw;
                     float ms = 0.f;
@@ -151,6 +161,15 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
                         break;
                     }
                 }
+            }
+            // the tiled sweep, kept unless a shape above is faster (it saves the cycle launches besides)
+            if (kind == kShapeSmooth && L.tparts > 0) {
+                LaunchShape tl;
+                L.shape[fp64][kind] = tl;
+                float ms = 0.f;
+                e = time_kernel<T>(c, L, kind, R, reps, e0, e1, &ms);
+                if (e != cudaSuccess) { L.shape[fp64][kind] = before; break; }
+                if (ms <= best_ms) { best = tl; best_ms = ms; }
             }
             L.shape[fp64][kind] = best;
             L.tuned_ms[fp64][kind] = best_ms;
@@ -188,12 +207,12 @@ int tune_cache_save(const char *path) {
     FILE *f = std::fopen(path, "w");
     if (!f) return 1;
     std::lock_guard<std::mutex> lk(g_mu);
-    std::fprintf(f, "# device fp64 kind lanes rows nnz threads_per_row threads_per_block [sweep_grid]\n");
+    std::fprintf(f, "# device fp64 kind lanes rows nnz threads_per_row threads_per_block [sweep_grid, -1: tiled sweep]\n");
     for (const auto &kv : g_cache) {
         const Key &k = kv.first;
         std::fprintf(f, "%s %d %d %d %lld %lld %d %d %d\n", std::get<0>(k).c_str(), std::get<1>(k), std::get<2>(k),
                      std::get<3>(k), (long long)std::get<4>(k), (long long)std::get<5>(k), kv.second.tpr,
-                     kv.second.tpb, kv.second.grid);
+                     kv.second.tpb, kv.second.tile && std::get<2>(k) == kShapeSmooth ? -1 : kv.second.grid);
     }
     return std::fclose(f) == 0 ? 0 : 1;
 }
@@ -210,7 +229,7 @@ int tune_cache_load(const char *path) {
         long long n, nnz;
         const int got = std::sscanf(line, "%255s %d %d %d %lld %lld %d %d %d", name, &fp64, &kind, &R, &n, &nnz, &tpr,
                                     &tpb, &grid);
-        if ((got != 8 && got != 9) || grid < 0 ||
+        if ((got != 8 && got != 9) || grid < -1 || (grid == -1 && kind != kShapeSmooth) ||
             (fp64 != 0 && fp64 != 1) || (kind != 0 && kind != 1) || (tpr != 4 && tpr != 8 && tpr != 16) ||
             tpb < 32 || (tpb > 512 && !(tpb == kSweepShapeTpb && tpr == 4 && kind == kShapeSmooth)) || tpb % 32 != 0) {
             bad = 1;
@@ -219,7 +238,8 @@ int tune_cache_load(const char *path) {
         LaunchShape sh;
         sh.tpr = tpr;
         sh.tpb = tpb;
-        sh.grid = tpb == kSweepShapeTpb ? grid : 0;
+        sh.grid = tpb == kSweepShapeTpb && grid > 0 ? grid : 0;
+        sh.tile = grid == -1;   // (a level without a plan runs the colour launches of the shape)
         g_cache[Key{std::string(name), fp64, kind, R, (int64_t)n, (int64_t)nnz}] = sh;
     }
     std::fclose(f);
