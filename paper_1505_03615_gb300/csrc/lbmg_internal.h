@@ -12,7 +12,7 @@ namespace lbmg {
 
 constexpr int kNQ = 4;            // Gauss-Legendre points per direction of the collapsed triangle rule
 constexpr int kMaxCoarse = 2048;  // largest coarsest level factored densely
-constexpr int kNormBlocks = 256;  // partial sums of the two-pass norm reduction
+constexpr int kNormBlocks = 608;  // partial sums of the two-pass norm reduction (four blocks per SM)
 
 // Launch shape of the row-parallel kernels (Gauss-Seidel colour sweep, residual):
 // tpr threads share one matrix row (4, 8 or 16), tpb threads per block (128-512).  With

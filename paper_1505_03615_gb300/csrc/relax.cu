@@ -44,6 +44,22 @@ __device__ __forceinline__ void load_x(const T *p, T (&v)[R]) {
     for (int r = 0; r < R; r++) v[r] = p[r];
 }
 
+template <>
+__device__ __forceinline__ void load_x<float, 4>(const float *p, float (&v)[4]) {
+    const float4 q = *reinterpret_cast<const float4 *>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+template <>
+__device__ __forceinline__ void load_x<double, 2>(const double *p, double (&v)[2]) {
+    const double2 q = *reinterpret_cast<const double2 *>(p);
+    v[0] = q.x; v[1] = q.y;
+}
+template <>
+__device__ __forceinline__ void load_x<double, 4>(const double *p, double (&v)[4]) {
+    const double2 q0 = reinterpret_cast<const double2 *>(p)[0], q1 = reinterpret_cast<const double2 *>(p)[1];
+    v[0] = q0.x; v[1] = q0.y; v[2] = q1.x; v[3] = q1.y;
+}
+
 // The static part of a matrix row (pattern and values) is loaded before the
 // kernel waits for its predecessor: each of the G threads of a row keeps its first
 // P entries in registers, so after the wait only the x gathers remain.
@@ -94,6 +110,41 @@ __device__ __forceinline__ void group_sum(T (&acc)[R]) {
     for (int o = G / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int r = 0; r < R; r++) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o, G);
+}
+
+// sums of the components over a warp, halved across its lanes so that an FP64 sum takes 6 additions of 4
+// components instead of 20 (GB300's FP64 pipe takes 64 cycles a warp instruction): one lane per component
+// returns its sum and the component in comp, the others -1
+template <class T, int R>
+__device__ __forceinline__ T warp_sum(const T (&a)[R], int lane, int &comp) {
+    constexpr unsigned kFull = 0xffffffffu;
+    T v;
+    int from;   // first of the butterfly steps left
+    if constexpr (R == 4) {
+        const bool hi = lane & 16, odd = lane & 8;
+        T a0 = hi ? a[2] : a[0], a1 = hi ? a[3] : a[1];
+        const T g0 = hi ? a[0] : a[2], g1 = hi ? a[1] : a[3];
+        a0 += __shfl_xor_sync(kFull, g0, 16);
+        a1 += __shfl_xor_sync(kFull, g1, 16);
+        const T give = odd ? a0 : a1;
+        v = (odd ? a1 : a0) + __shfl_xor_sync(kFull, give, 8);
+        from = 4;
+        comp = (lane & 7) == 0 ? lane >> 3 : -1;
+    } else if constexpr (R == 2) {
+        const bool hi = lane & 16;
+        const T give = hi ? a[0] : a[1];
+        v = (hi ? a[1] : a[0]) + __shfl_xor_sync(kFull, give, 16);
+        from = 8;
+        comp = (lane & 15) == 0 ? lane >> 4 : -1;
+    } else {
+        v = a[0];
+        from = 16;
+        comp = lane == 0 ? 0 : -1;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (o <= from) v += __shfl_xor_sync(kFull, v, o);
+    return v;
 }
 
 template <class T, int R, int G>
@@ -230,27 +281,31 @@ void launch_jacobi_update(const DevLevel &L, const T *dinv, const T *r, T *x, T 
 }
 
 // b_c[J] = sum over fine children i of J of r_f[i] / #parents(i); x_c[J] = 0 when x_c is given.
-// The first kPreChildren entries of the static child list are loaded before the
-// grid-dependency wait, so after it only the residual gathers remain, all in flight
-// together.
-constexpr int kPreChildren = 16;
+// Eight lanes share a coarse row (14 children on average, up to 60 or so): neighbouring lanes read
+// neighbouring list entries, and a row's gathers are three per lane and all in flight together.  One thread
+// per row read the lists a row apart and chained its gathers: 46 us from 927k to 232k rows (four FP32
+// components) and 8 to 11 us on levels of some thousand rows, where the chain was the time.  Each lane's
+// first kPreChildren entries are loaded before the grid-dependency wait.  The components' sums are halved
+// across the lanes: lane 4 h + 2 o of a row ends with component 2 h + o.
+constexpr int kPreChildren = 3;
 
 template <class T, int R>
-__global__ void restrict_kernel(int nc, const int *__restrict__ crp, const uint32_t *__restrict__ cch,
-                                const T *__restrict__ rf, T *__restrict__ bc, T *__restrict__ xc,
-                                const T *__restrict__ dinv, int c1) {
-    const int J = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) restrict_kernel(int nc, const int *__restrict__ crp,
+                                                       const uint32_t *__restrict__ cch, const T *__restrict__ rf,
+                                                       T *__restrict__ bc, T *__restrict__ xc,
+                                                       const T *__restrict__ dinv, int c1) {
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int J = tid >> 3, l = tid & 7;
     const bool active = J < nc;
     int k0 = 0, k1 = 0;
     uint32_t e[kPreChildren];
-    if (active) { k0 = __ldg(crp + J); k1 = __ldg(crp + J + 1); }
+    if (active) { k0 = __ldg(crp + J) + l; k1 = __ldg(crp + J + 1); }
     // colour 0 (rows [0, c1)) of the first sweep, fused: its inverse diagonal
     const T d = (active && dinv && J < c1) ? __ldg(dinv + J) : T(0);
 #pragma unroll
-    for (int u = 0; u < kPreChildren; u++) e[u] = k0 + u < k1 ? __ldg(cch + k0 + u) : 0u;
+    for (int u = 0; u < kPreChildren; u++) e[u] = k0 + 8 * u < k1 ? __ldg(cch + k0 + 8 * u) : 0u;
     grid_dep_wait();
     grid_dep_launch();
-    if (!active) return;
     T acc[R];
 #pragma unroll
     for (int r = 0; r < R; r++) acc[r] = T(0);
@@ -263,27 +318,47 @@ __global__ void restrict_kernel(int nc, const int *__restrict__ crp, const uint3
     };
 #pragma unroll
     for (int u = 0; u < kPreChildren; u++)
-        if (k0 + u < k1) child(e[u]);
-    for (int k = k0 + kPreChildren; k < k1; k++) child(__ldg(cch + k));
-#pragma unroll
-    for (int r = 0; r < R; r++) bc[(size_t)J * R + r] = acc[r];
-    if (xc) {
-        if (dinv && J < c1) {
-            // the colour kernels' step x = x + (b - A x) / a_ii with x = 0 (so A x = +0): 0 + b d
-#pragma unroll
-            for (int r = 0; r < R; r++) xc[(size_t)J * R + r] = T(0) + (acc[r] - T(0)) * d;
-        } else {
-#pragma unroll
-            for (int r = 0; r < R; r++) xc[(size_t)J * R + r] = T(0);
-        }
+        if (k0 + 8 * u < k1) child(e[u]);
+    for (int k = k0 + 8 * kPreChildren; k < k1; k += 8) child(__ldg(cch + k));
+    constexpr unsigned kFull = 0xffffffffu;
+    T v;
+    int comp;
+    bool writes;
+    if constexpr (R == 4) {
+        const bool hi = l & 4, odd = l & 2;
+        T a0 = hi ? acc[2] : acc[0], a1 = hi ? acc[3] : acc[1];
+        const T g0 = hi ? acc[0] : acc[2], g1 = hi ? acc[1] : acc[3];
+        a0 += __shfl_xor_sync(kFull, g0, 4);
+        a1 += __shfl_xor_sync(kFull, g1, 4);
+        const T give = odd ? a0 : a1;
+        v = (odd ? a1 : a0) + __shfl_xor_sync(kFull, give, 2);
+        comp = l >> 1;
+        writes = (l & 1) == 0;
+    } else if constexpr (R == 2) {
+        const bool hi = l & 4;
+        const T give = hi ? acc[0] : acc[1];
+        v = (hi ? acc[1] : acc[0]) + __shfl_xor_sync(kFull, give, 4);
+        v += __shfl_xor_sync(kFull, v, 2);
+        comp = l >> 2;
+        writes = (l & 3) == 0;
+    } else {
+        v = acc[0] + __shfl_xor_sync(kFull, acc[0], 4);
+        v += __shfl_xor_sync(kFull, v, 2);
+        comp = 0;
+        writes = l == 0;
     }
+    v += __shfl_xor_sync(kFull, v, 1);
+    if (!active || !writes) return;
+    bc[(size_t)J * R + comp] = v;
+    // the colour kernels' step x = x + (b - A x) / a_ii with x = 0 (so A x = +0): 0 + b d
+    if (xc) xc[(size_t)J * R + comp] = dinv && J < c1 ? T(0) + (v - T(0)) * d : T(0);
 }
 
 template <class T>
 void launch_restrict(const DevLevel &Lc, const T *rf, T *bc, int R, cudaStream_t s, T *xc, Chain *ch,
                      bool first_colour) {
     if (Lc.n == 0) return;
-    const unsigned blocks = (unsigned)((Lc.n + 255) / 256);
+    const unsigned blocks = (unsigned)(((int64_t)Lc.n * 8 + 255) / 256);
     auto k = R == 1 ? restrict_kernel<T, 1> : R == 2 ? restrict_kernel<T, 2> : restrict_kernel<T, 4>;
     const T *dinv = first_colour && xc ? (sizeof(T) == 4 ? (const T *)Lc.dinv32 : (const T *)Lc.dinv64) : nullptr;
     klaunch(k, blocks, 256u, 0, s, ch, Lc.n, Lc.crp, Lc.cch, rf, bc, xc, dinv, dinv ? Lc.cs[1] : 0);
@@ -298,8 +373,10 @@ __global__ void prolong_add_kernel(int nf, const int *__restrict__ par, const in
     int np = 0, p[8];
     if (active) {
         np = 1 << __ldg(npl2 + i);
-#pragma unroll
-        for (int q = 0; q < 8; q++) p[q] = q < np ? __ldg(par + 8 * (size_t)i + q) : 0;
+        const int4 p0 = __ldg(reinterpret_cast<const int4 *>(par + 8 * (size_t)i));
+        const int4 p1 = __ldg(reinterpret_cast<const int4 *>(par + 8 * (size_t)i) + 1);   // the same 32 bytes
+        p[0] = p0.x; p[1] = p0.y; p[2] = p0.z; p[3] = p0.w;
+        p[4] = p1.x; p[5] = p1.y; p[6] = p1.z; p[7] = p1.w;
     }
     grid_dep_wait();
     grid_dep_launch();
@@ -329,34 +406,42 @@ void launch_prolong_add(const DevLevel &Lf, const T *xc, T *xf, int R, cudaStrea
     klaunch(k, blocks, 256u, 0, s, ch, Lf.ns, Lf.par, Lf.npl2, xc, xf);
 }
 
-// x = inv * b on every coarsest block of a level (one block per mesh), one warp per row
+// x = inv * b on every coarsest block of a level (one per mesh), one warp per row, kCoarseRows rows per
+// thread block, so that the rows spread over the SMs: in one thread block the FP64 product of 124 rows kept
+// one SM's FP64 pipe busy for 73 us of a cycle.  The row of the inverse, static during a solve, is loaded
+// before the grid-dependency wait (its first 32 kCoarsePre entries).
+constexpr int kCoarseRows = 4, kCoarsePre = 5;
+
 template <class T, int R>
-__global__ void coarse_apply_kernel(const int *__restrict__ cblk, const T *__restrict__ inv, const T *__restrict__ b,
-                                    T *__restrict__ x) {
-    const int *cb = cblk + 5 * blockIdx.x;
+__global__ void __launch_bounds__(32 * kCoarseRows) coarse_apply_kernel(const int *__restrict__ cblk, int chunks,
+                                                                        const T *__restrict__ inv,
+                                                                        const T *__restrict__ b, T *__restrict__ x) {
+    const int *cb = cblk + 5 * (blockIdx.x / chunks);
     const int row0 = cb[2], n = cb[3];
-    const T *M = inv + cb[4];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, row = (int)(blockIdx.x % chunks) * kCoarseRows + (int)(threadIdx.x >> 5);
+    const T *M = inv + cb[4] + (size_t)row * n;
+    T a[kCoarsePre];
+#pragma unroll
+    for (int u = 0; u < kCoarsePre; u++) a[u] = row < n && lane + 32 * u < n ? __ldg(M + lane + 32 * u) : T(0);
     grid_dep_wait();
     grid_dep_launch();
-    for (int row = warp; row < n; row += nw) {
-        T acc[R];
+    if (row >= n) return;
+    T acc[R];
 #pragma unroll
-        for (int r = 0; r < R; r++) acc[r] = T(0);
-        for (int j = lane; j < n; j += 32) {
-            const T a = M[(size_t)row * n + j];
+    for (int r = 0; r < R; r++) acc[r] = T(0);
+    auto term = [&](int j, T av) {
+        T v[R];
+        load_x<T, R>(b + (size_t)(row0 + j) * R, v);
 #pragma unroll
-            for (int r = 0; r < R; r++) acc[r] = fma(a, b[(size_t)(row0 + j) * R + r], acc[r]);
-        }
+        for (int r = 0; r < R; r++) acc[r] = fma(av, v[r], acc[r]);
+    };
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int r = 0; r < R; r++) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
-        if (lane == 0) {
-#pragma unroll
-            for (int r = 0; r < R; r++) x[(size_t)(row0 + row) * R + r] = acc[r];
-        }
-    }
+    for (int u = 0; u < kCoarsePre; u++)
+        if (lane + 32 * u < n) term(lane + 32 * u, a[u]);
+    for (int j = lane + 32 * kCoarsePre; j < n; j += 32) term(j, __ldg(M + j));
+    int comp;
+    const T v = warp_sum<T, R>(acc, lane, comp);
+    if (comp >= 0) x[(size_t)(row0 + row) * R + comp] = v;
 }
 
 template <class T>
@@ -364,8 +449,11 @@ void launch_coarse_apply(const Ctx &c, const DevLevel &L, const T *inv, const T 
                          Chain *ch) {
     if (L.ncb == 0) return;
     const int *cb = c.cblk + 5 * L.cb0;
+    int n = 1;
+    for (int k = L.cb0; k < L.cb0 + L.ncb; k++) n = std::max(n, c.cblk_host[5 * (size_t)k + 3]);
+    const int chunks = (n + kCoarseRows - 1) / kCoarseRows;
     auto k = R == 1 ? coarse_apply_kernel<T, 1> : R == 2 ? coarse_apply_kernel<T, 2> : coarse_apply_kernel<T, 4>;
-    klaunch(k, (unsigned)L.ncb, 256u, 0, s, ch, cb, inv, b, x);
+    klaunch(k, (unsigned)(L.ncb * chunks), 32u * kCoarseRows, 0, s, ch, cb, chunks, inv, b, x);
 }
 
 // ---- coarsest-level dense FP64 Cholesky of A + eps Id, eps = 1e-12 mean diag ----
@@ -462,44 +550,56 @@ void launch_coarse_factor(const Ctx &c, const int *const *rps, const int *const 
 }
 
 // ---- per-right-hand-side sums of squares, two passes (deterministic) ----
+// the block's sum of each component: per warp, then over the warps; thread c < R returns component c
+template <int R>
+__device__ __forceinline__ double block_sum(const double (&acc)[R]) {
+    __shared__ double sh[8][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int comp;
+    const double v = warp_sum<double, R>(acc, lane, comp);
+    if (comp >= 0) sh[warp][comp] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < R)
+        for (int w = 0; w < 8; w++) t += sh[w][threadIdx.x];
+    return t;
+}
+
+// One round of blocks over the GPU, a row's components in one or two vector loads.  (256 blocks and scalar
+// loads took 38 us for 927k rows of four components, 30 MB.)
 template <int R>
 __global__ void __launch_bounds__(256) norm_partial_kernel(const double *__restrict__ v, int n, double *__restrict__ part) {
-    __shared__ double sh[256][R];
     grid_dep_wait();
     grid_dep_launch();
     double acc[R];
 #pragma unroll
     for (int r = 0; r < R; r++) acc[r] = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+#pragma unroll 4
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        double x[R];
+        load_x<double, R>(v + (size_t)i * R, x);
 #pragma unroll
-        for (int r = 0; r < R; r++) { const double x = v[(size_t)i * R + r]; acc[r] = fma(x, x, acc[r]); }
-#pragma unroll
-    for (int r = 0; r < R; r++) sh[threadIdx.x][r] = acc[r];
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-#pragma unroll
-            for (int r = 0; r < R; r++) sh[threadIdx.x][r] += sh[threadIdx.x + o][r];
-        __syncthreads();
+        for (int r = 0; r < R; r++) acc[r] = fma(x[r], x[r], acc[r]);
     }
-    if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = sh[0][threadIdx.x];
+    const double t = block_sum<R>(acc);
+    if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = t;
 }
 
-__global__ void __launch_bounds__(256) norm_final_kernel(const double *__restrict__ part, int nblocks, int R,
+// sum of the blocks' partials of component c, by warp c
+__device__ __forceinline__ double partials_sum(const double *__restrict__ part, int nblocks, int c, int lane) {
+    double acc[1] = {0.0};
+    for (int b = lane; b < nblocks; b += 32) acc[0] += part[b * 4 + c];
+    int comp;
+    return warp_sum<double, 1>(acc, lane, comp);
+}
+
+__global__ void __launch_bounds__(128) norm_final_kernel(const double *__restrict__ part, int nblocks, int R,
                                                          double *__restrict__ out) {
-    __shared__ double sh[256][4];
     grid_dep_wait();
     grid_dep_launch();
-    for (int r = 0; r < 4; r++) sh[threadIdx.x][r] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        for (int r = 0; r < R; r++) sh[threadIdx.x][r] += part[b * 4 + r];
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int r = 0; r < 4; r++) sh[threadIdx.x][r] += sh[threadIdx.x + o][r];
-        __syncthreads();
-    }
-    if (threadIdx.x < 4) out[threadIdx.x] = threadIdx.x < R ? sh[0][threadIdx.x] : 0.0;
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double v = c < R ? partials_sum(part, nblocks, c, lane) : 0.0;
+    if (lane == 0) out[c] = v;
 }
 
 // ---- conjugate gradients preconditioned by the V-cycle (per right-hand side lane) ----
@@ -507,23 +607,19 @@ __global__ void __launch_bounds__(256) norm_final_kernel(const double *__restric
 template <int R>
 __global__ void __launch_bounds__(256) dot_partial_kernel(const double *__restrict__ a, const double *__restrict__ b,
                                                           int n, double *__restrict__ part) {
-    __shared__ double sh[256][R];
     double acc[R];
 #pragma unroll
     for (int r = 0; r < R; r++) acc[r] = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+#pragma unroll 4
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        double x[R], y[R];
+        load_x<double, R>(a + (size_t)i * R, x);
+        load_x<double, R>(b + (size_t)i * R, y);
 #pragma unroll
-        for (int r = 0; r < R; r++) acc[r] = fma(a[(size_t)i * R + r], b[(size_t)i * R + r], acc[r]);
-#pragma unroll
-    for (int r = 0; r < R; r++) sh[threadIdx.x][r] = acc[r];
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-#pragma unroll
-            for (int r = 0; r < R; r++) sh[threadIdx.x][r] += sh[threadIdx.x + o][r];
-        __syncthreads();
+        for (int r = 0; r < R; r++) acc[r] = fma(x[r], y[r], acc[r]);
     }
-    if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = sh[0][threadIdx.x];
+    const double t = block_sum<R>(acc);
+    if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = t;
 }
 
 // one scalar step of lane r on the reduced value v (scalars sc, see pcg_scalar_kernel)
@@ -550,22 +646,12 @@ __device__ __forceinline__ void pcg_scalar_step(double *sc, int r, double v, int
 //   mode 1: s1 = v; beta = (s1 - s2) / rz, rz = s1  (Polak-Ribiere; 0 on the first step, rz = 0;
 //           a lane at rounding level, v <= kPcgStop * its first v, keeps beta = alpha = 0)
 //   mode 2: alpha = s1 / (p . A p), with v = p . q and q = -A p
-__global__ void pcg_scalar_kernel(const double *__restrict__ part, int nblocks, int R, double *__restrict__ sc,
-                                  int mode) {
-    __shared__ double sh[256][4];
-    for (int r = 0; r < 4; r++) sh[threadIdx.x][r] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        for (int r = 0; r < R; r++) sh[threadIdx.x][r] += part[b * 4 + r];
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int r = 0; r < 4; r++) sh[threadIdx.x][r] += sh[threadIdx.x + o][r];
-        __syncthreads();
-    }
-    if (threadIdx.x >= R) return;
-    const int r = threadIdx.x;
-    const double v = sh[0][r];
-    pcg_scalar_step(sc, r, v, mode);
+__global__ void __launch_bounds__(128) pcg_scalar_kernel(const double *__restrict__ part, int nblocks, int R,
+                                                         double *__restrict__ sc, int mode) {
+    const int r = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (r >= R) return;
+    const double v = partials_sum(part, nblocks, r, lane);
+    if (lane == 0) pcg_scalar_step(sc, r, v, mode);
 }
 
 // p = z + beta p
@@ -700,7 +786,7 @@ void launch_pcg_dot(const double *a, const double *b, int n, int R, double *part
     if (R == 1) dot_partial_kernel<1><<<kNormBlocks, 256, 0, s>>>(a, b, n, part);
     else if (R == 2) dot_partial_kernel<2><<<kNormBlocks, 256, 0, s>>>(a, b, n, part);
     else dot_partial_kernel<4><<<kNormBlocks, 256, 0, s>>>(a, b, n, part);
-    pcg_scalar_kernel<<<1, 256, 0, s>>>(part, kNormBlocks, R, sc, mode);
+    pcg_scalar_kernel<<<1, 128, 0, s>>>(part, kNormBlocks, R, sc, mode);
 }
 void launch_pcg_direction(const double *z, double *p, const double *sc, int n, int R, cudaStream_t s) {
     const int64_t m = (int64_t)n * R;
@@ -715,7 +801,7 @@ void launch_pcg_update(double *x, double *r, const double *p, const double *q, c
 void launch_norms(const double *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch) {
     auto k = R == 1 ? norm_partial_kernel<1> : R == 2 ? norm_partial_kernel<2> : norm_partial_kernel<4>;
     klaunch(k, (unsigned)kNormBlocks, 256u, 0, s, ch, v, n, part);
-    klaunch(norm_final_kernel, 1u, 256u, 0, s, ch, (const double *)part, (int)kNormBlocks, R, out);
+    klaunch(norm_final_kernel, 1u, 128u, 0, s, ch, (const double *)part, (int)kNormBlocks, R, out);
 }
 
 // ---- layout and elementwise kernels ----
