@@ -247,15 +247,18 @@ template <> struct P<double> {
     static const double *inv(Ctx &c) { return c.cinv64; }
 };
 
-// whether the level's sweeps run in the tiled kernel: it has a plan and no other launch shape was chosen
+// whether the level's sweeps run in the tiled kernel: it has a plan, no other launch shape was chosen, and
+// its tiles are resident at once
 template <class T>
-bool tiled(const Ctx &c, const DevLevel &L) {
-    return c.smoother == LBMG_GS_COLOURED && L.tparts > 0 && L.shape[sizeof(T) == 8][kShapeSmooth].tile;
+bool tiled(const Ctx &c, const DevLevel &L, int R) {
+    const bool f64 = sizeof(T) == 8;
+    return c.smoother == LBMG_GS_COLOURED && L.tparts > 0 && L.tonce[f64][R >> 1] && L.shape[f64][kShapeSmooth].tile;
 }
 
 template <class T>
-void enqueue_smooth(Ctx &c, DevLevel &L, int R, int sweeps, bool forward, cudaStream_t s, Chain *ch, int skip = 0) {
-    if (tiled<T>(c, L)) {
+void enqueue_smooth(Ctx &c, DevLevel &L, int R, int sweeps, bool forward, cudaStream_t s, Chain *ch, int skip = 0,
+                    bool from_zero = false) {
+    if (tiled<T>(c, L, R)) {
         // from one vector to the other and back; the rows behind ns keep their place in x
         TileVec<T> v{P<T>::x(L), P<T>::y(L)};
         for (int sw = 0; sw < sweeps; sw++)
@@ -271,7 +274,7 @@ void enqueue_smooth(Ctx &c, DevLevel &L, int R, int sweeps, bool forward, cudaSt
             if (ch) ch->cut();
         }
     } else {
-        launch_sweeps<T>(c, L, sweeps, forward, P<T>::A(L), P<T>::dinv(L), P<T>::b(L), P<T>::x(L), R, s, ch, skip);
+        launch_sweeps<T>(c, L, sweeps, forward, P<T>::A(L), P<T>::dinv(L), P<T>::b(L), P<T>::x(L), R, s, ch, skip, from_zero);
     }
 }
 
@@ -288,6 +291,15 @@ inline void record(cudaEvent_t e, cudaStream_t s, Chain *ch) {
 // Every coarser correction is zeroed by the restriction that fills its right-hand
 // side, so the kernels of the cycle follow one another with no memset between
 // them and run as one chain of dependent launches.
+// whether a V-cycle from zero on level d reads nothing of its x before it has written it
+template <class T>
+bool top_from_zero(const Ctx &c, int d, int R) {
+    const DevLevel &L = c.lev[d];
+    return c.gamma == 1 && !c.coarse_smooth && c.nu1 > 0 && d > c.d0 &&
+           ((tiled<T>(c, L, R) && c.nu2 > 0) ||
+            (c.smoother == LBMG_GS_COLOURED && !tiled<T>(c, L, R) && sweeps_from_zero<T>(L)));
+}
+
 // Tiled levels take a launch or two per sweep, the residual with the last sweep down, the prolongation in
 // the first one up (timed: the events bracket these too).
 // zero: e is zero on entry (the tiled finest level does not read it then).
@@ -305,7 +317,7 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
     }
     int skip = 0;   // colour steps of the next level's first sweep that its restriction did
     TileVec<T> vec[kMaxDepth + 1];
-    auto tile = [&](int d) { return c.nu1 > 0 && c.nu2 > 0 && tiled<T>(c, c.lev[d]); };
+    auto tile = [&](int d) { return c.nu1 > 0 && c.nu2 > 0 && tiled<T>(c, c.lev[d], R); };
     for (int d = top; d > dn; d--) {
         DevLevel &L = c.lev[d], &Lc = c.lev[d - 1];
         launch_coarse_apply<T>(c, L, P<T>::inv(c), P<T>::b(L), P<T>::x(L), R, s, ch);
@@ -325,7 +337,7 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
                 launch_tile_sweep<T>(c, L, true, v, P<T>::b(L), q + 1 == c.nu1 ? P<T>::r(L) : (T *)nullptr, R, s, ch);
             if (timed && d == top) record(c.ev_smooth[1], s, ch);
         } else {
-            enqueue_smooth<T>(c, L, R, c.nu1, true, s, ch, skip);
+            enqueue_smooth<T>(c, L, R, c.nu1, true, s, ch, skip, d == top && zero_start && top_from_zero<T>(c, d, R));
             if (timed && d == top) record(c.ev_smooth[1], s, ch);
             launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch);
         }
@@ -348,8 +360,13 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
         DevLevel &L = c.lev[d];
         if (tile(d)) {
             TileVec<T> &v = vec[d];
-            v.xc = P<T>::x(c.lev[d - 1]);
-            v.prolong = (1u << L.tparts) - 1u;
+            // on large levels a pass of its own: the rims would read 1.5 times the parents
+            if (L.ns > kTileProlong) {
+                launch_prolong_add<T>(L, P<T>::x(c.lev[d - 1]), v.cur ? v.y : v.x, R, s, ch);
+            } else {
+                v.xc = P<T>::x(c.lev[d - 1]);
+                v.prolong = (1u << L.tparts) - 1u;
+            }
             if (timed && d == top) record(c.ev_smooth[2], s, ch);
             for (int q = 0; q < c.nu2; q++)
                 launch_tile_sweep<T>(c, L, false, v, P<T>::b(L), (T *)nullptr, R, s, ch);
@@ -410,11 +427,22 @@ Chain make_chain(const Ctx &c, cudaStream_t s) {
     return ch;
 }
 
-// the mixed V-cycle iteration keeps its iterate as an FP32 pair (c.xs_hi + c.xs_lo, updated by
+// the mixed V-cycle iteration keeps its iterate as FP32 pairs (c.xs_pair, updated by
 // an FP32 two-sum) and forms the outer residual from it; c.xs holds it in FP64 only before and
 // after the solve (split at the start, joined at the end)
 inline bool pair_iterate(const Ctx &c, int precision, bool pcg) {
     return precision == LBMG_MIXED && !pcg && c.lev[c.D].pk_v2 != nullptr;
+}
+
+// what a mixed iteration with the iterate as a pair finds prepared (by the one before, or before the first):
+// the right-hand side of the solve as three FP32 numbers, the residual in FP32 (F.b32) and, where the cycle
+// reads it, a zero start
+void enqueue_pair_start(Ctx &c, int R, cudaStream_t s) {
+    DevLevel &F = c.lev[c.D];
+    const int64_t m = (int64_t)F.n * R;
+    launch_split(c.xs, c.xs_pair, F.n, R, s);
+    launch_split3(c.bs, c.bs3, m, s);
+    if (!c.learned_on) launch_to_float(c.rs, F.b32, m, s, top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32);
 }
 
 // one defect-correction step: x += Vcycle(r); r = b - A x; norms(r)
@@ -424,15 +452,22 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
     const int64_t m = (int64_t)F.n * R;
     Chain ch = make_chain(c, s);
     if (precision == LBMG_MIXED) {
+        const bool pairs = pair_iterate(c, precision, false);
         if (c.learned_on) learned_enqueue(c, R, precision, s, &ch);   // the cycle starts from the correction
-        else launch_to_float(c.rs, F.b32, m, s, F.x32, &ch);
+        else if (!pairs) launch_to_float(c.rs, F.b32, m, s, F.x32, &ch);
         enqueue_cycle<float>(c, R, s, timed, &ch, !c.learned_on);
         // x += e, and the outer residual with FP64 values carried as FP32 pairs (GB300's FP64
         // rate would bound an FP64 residual of the finest level)
-        if (pair_iterate(c, precision, false)) {
-            launch_add_pair(F.x32, c.xs_hi, c.xs_lo, m, s, &ch);
-            launch_packed_residual_split(F, c.bs, c.xs_hi, c.xs_lo, c.rs, R, s, &ch);
-            launch_norms(c.rs, F.n, R, c.norm_part, c.norm_out, s, &ch);
+        if (pairs) {
+            launch_add_pair(F.x32, c.xs_pair, F.n, R, s, &ch);
+            if (c.learned_on) {   // the correction reads the residual itself
+                launch_packed_residual_split(F, c.bs, c.xs_pair, c.rs, R, s, &ch);
+                launch_norms(c.rs, F.n, R, c.norm_part, c.norm_out, s, &ch);
+            } else {
+                launch_packed_outer(F, c.bs3, c.xs_pair, F.b32, top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32, R,
+                                    c.lanes, s, &ch);
+                launch_norms32(F.b32, F.n, R, c.norm_part, c.norm_out, s, &ch);
+            }
             return;
         }
         launch_add_float(c.xs, F.x32, m, s, &ch);
@@ -441,7 +476,7 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
             learned_enqueue(c, R, precision, s, &ch);
         } else {
             cudaMemcpyAsync(F.b64, c.rs, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
-            cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
+            if (!top_from_zero<double>(c, c.D, R)) cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
         }
         enqueue_cycle<double>(c, R, s, timed, &ch, !c.learned_on);
         launch_add_double(c.xs, F.x64, m, s);
@@ -455,8 +490,8 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
 // (the product of the outer residual), else in FP64
 void enqueue_pcg_product(Ctx &c, DevLevel &F, int R, int precision, int64_t m, cudaStream_t s) {
     if (precision == LBMG_MIXED && F.pk_v2) {
-        launch_split(c.pcg_p, c.xs_hi, c.xs_lo, m, s);
-        if (launch_packed_residual_split(F, c.pcg_zero, c.xs_hi, c.xs_lo, c.pcg_q, R, s, nullptr)) return;
+        launch_split(c.pcg_p, c.xs_pair, F.n, R, s);
+        if (launch_packed_residual_split(F, c.pcg_zero, c.xs_pair, c.pcg_q, R, s, nullptr)) return;
     }
     launch_residual<double>(F, F.A64, c.pcg_zero, c.pcg_p, c.pcg_q, R, s);
 }
@@ -471,12 +506,12 @@ void enqueue_pcg_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool ti
     launch_pcg_dot(c.rs, c.pcg_z, F.n, R, c.pcg_part, c.pcg_s, 0, s);
     Chain ch = make_chain(c, s);
     if (precision == LBMG_MIXED) {
-        launch_to_float(c.rs, F.b32, m, s, F.x32, &ch);
+        launch_to_float(c.rs, F.b32, m, s, top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32, &ch);
         enqueue_cycle<float>(c, R, s, timed, &ch);
         to_double_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(F.x32, c.pcg_z, m);
     } else {
         cudaMemcpyAsync(F.b64, c.rs, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
-        cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
+        if (!top_from_zero<double>(c, c.D, R)) cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
         enqueue_cycle<double>(c, R, s, timed, &ch);
         cudaMemcpyAsync(c.pcg_z, F.x64, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
     }
@@ -497,12 +532,12 @@ void enqueue_pcg_batch_iteration(Ctx &c, int R, int precision, cudaStream_t s) {
     launch_inst_pcg_scalar(c.item_start, c.ninst, R, c.item_part, c.pcg_si, 0, c.inst_norm, c.pcg_tol, s);
     Chain ch = make_chain(c, s);
     if (precision == LBMG_MIXED) {
-        launch_to_float(c.rs, F.b32, m, s, F.x32, &ch);
+        launch_to_float(c.rs, F.b32, m, s, top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32, &ch);
         enqueue_vcycle<float>(c, R, s, false, &ch);
         to_double_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(F.x32, c.pcg_z, m);
     } else {
         cudaMemcpyAsync(F.b64, c.rs, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
-        cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
+        if (!top_from_zero<double>(c, c.D, R)) cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
         enqueue_vcycle<double>(c, R, s, false, &ch);
         cudaMemcpyAsync(c.pcg_z, F.x64, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
     }
@@ -719,6 +754,11 @@ int build_tiles(lbmg_handle h, const HostLevel &hl, DevLevel &L, int sms) {
     LBMG_TRY(h->alloc(&L.y32, 4 * (size_t)L.n));
     L.tparts = parts;
     L.tfused = fused;
+    for (int p = 0; p < 2; p++)
+        for (int r = 0; r < 3; r++) {
+            L.tonce[p][r] = true;
+            for (const Job &j : jobs) L.tonce[p][r] = L.tonce[p][r] && j.t->at_once[p][r];
+        }
     return LBMG_OK;
 }
 
@@ -889,8 +929,8 @@ int upload_hierarchy(lbmg_handle h) {
     LBMG_TRY(h->alloc(&c.xs, 4 * nD));
     LBMG_TRY(h->alloc(&c.bs, 4 * nD));
     LBMG_TRY(h->alloc(&c.rs, 4 * nD));
-    LBMG_TRY(h->alloc(&c.xs_hi, 4 * nD));
-    LBMG_TRY(h->alloc(&c.xs_lo, 4 * nD));
+    LBMG_TRY(h->alloc(&c.xs_pair, 8 * nD));
+    LBMG_TRY(h->alloc(&c.bs3, 4 * nD));
     LBMG_TRY(h->alloc(&c.norm_part, 4 * (size_t)kNormBlocks));
     LBMG_TRY(h->alloc(&c.pcg_z, 4 * nD));
     LBMG_TRY(h->alloc(&c.pcg_p, 4 * nD));
@@ -1356,7 +1396,7 @@ static int solve_cond(lbmg_handle h, cudaGraphExec_t exec, const double *rd, con
     launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s);
     const size_t m = (size_t)Fl.n * R;
     const bool pairs = pair_iterate(c, precision, pcg);
-    if (pairs) launch_split(c.xs, c.xs_hi, c.xs_lo, (int64_t)m, s);
+    if (pairs) enqueue_pair_start(c, R, s);
     if (pcg) {
         LBMG_CK(cudaMemsetAsync(c.pcg_z, 0, m * sizeof(double), s));
         LBMG_CK(cudaMemsetAsync(c.pcg_p, 0, m * sizeof(double), s));
@@ -1373,7 +1413,7 @@ static int solve_cond(lbmg_handle h, cudaGraphExec_t exec, const double *rd, con
         launch_norms(c.rs, Fl.n, R, c.norm_part, c.norm_out, s);
     }
     LBMG_CK(cudaGraphLaunch(exec, s));
-    if (pairs) launch_join(c.xs_hi, c.xs_lo, c.xs, (int64_t)m, s);
+    if (pairs) launch_join(c.xs_pair, c.xs, Fl.n, R, s);
     launch_unpack(c.xs, Fl.n, nrhs, R, xout, s, c.fperm);
     LBMG_CK(cudaEventRecord(c.ev1, s));
     LBMG_CK(cudaMemcpyAsync(c.h_ctl, c.ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, s));
@@ -1601,7 +1641,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
     launch_pack(xin, Fl.n, nrhs, R, c.xs, s, c.fperm);
     launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s);
     const bool pairs = pair_iterate(c, precision, pcg);
-    if (pairs) launch_split(c.xs, c.xs_hi, c.xs_lo, (int64_t)Fl.n * R, s);
+    if (pairs) enqueue_pair_start(c, R, s);
     if (pcg) {
         LBMG_CK(cudaMemsetAsync(c.pcg_z, 0, (size_t)Fl.n * R * sizeof(double), s));
         LBMG_CK(cudaMemsetAsync(c.pcg_p, 0, (size_t)Fl.n * R * sizeof(double), s));
@@ -1674,7 +1714,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
         }
         cycles = max_cycles;
     }
-    if (pairs) launch_join(c.xs_hi, c.xs_lo, c.xs, (int64_t)Fl.n * R, s);
+    if (pairs) launch_join(c.xs_pair, c.xs, Fl.n, R, s);
     launch_unpack(c.xs, Fl.n, nrhs, R, xout, s, c.fperm);
     LBMG_CK(cudaEventRecord(c.ev1, s));
     LBMG_TRY(finish_output(x, xout, cnt, host_out, s, &h->syncs));
@@ -1797,8 +1837,8 @@ int lbmg_residual_split(lbmg_handle h, int d, const double *rhs, const double *x
     launch_pack(bd, L.n, nrhs, R, L.b64, s);
     LBMG_TRY(input_ptr(h, x, cnt, 1, s, &xd));
     launch_pack(xd, L.n, nrhs, R, L.x64, s);
-    launch_split(L.x64, L.x32, L.r32, (int64_t)L.n * R, s);   // the level's FP32 vectors as scratch
-    launch_packed_residual_split(L, L.b64, L.x32, L.r32, L.r64, R, s, nullptr);
+    launch_split(L.x64, reinterpret_cast<float *>(L.x64), L.n, R, s);   // in place
+    launch_packed_residual_split(L, L.b64, reinterpret_cast<const float *>(L.x64), L.r64, R, s, nullptr);
     LBMG_TRY(output_ptr(h, r, cnt, 0, &rd, &host_out));
     launch_unpack(L.r64, L.n, nrhs, R, rd, s);
     return finish_output(r, rd, cnt, host_out, s);
@@ -1893,7 +1933,7 @@ int lbmg_launch_counts(lbmg_handle h, int precision, int *assemble, int *project
         for (int d = bottom + 1; d <= c.D; d++) {   // sweeps, residual, restriction, prolongation
             const DevLevel &L = c.lev[d];
             if (c.nu1 > 0 && c.nu2 > 0 && c.smoother != LBMG_JACOBI && L.tparts > 0 &&
-                L.shape[precision == LBMG_FP64][kShapeSmooth].tile) {   // sweeps, residual, restriction
+                L.tonce[precision == LBMG_FP64][2] && L.shape[precision == LBMG_FP64][kShapeSmooth].tile) {   // sweeps, residual, restriction
                 cyc += (c.nu1 + c.nu2) * L.tparts + (L.tfused ? 0 : 1) + 1 + (L.ncb > 0);
                 continue;
             }

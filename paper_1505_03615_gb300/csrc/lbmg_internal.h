@@ -79,6 +79,7 @@ struct TileDev {
     int ntile = 0, nsteps = 0, maxloc = 0, maxcomp = 0, maxgrp = 0, maxquads = 0;
     int64_t groups = 0, quads = 0;
     int ring[2][3] = {{0}};                // [FP64][R = 1, 2, 4] groups in flight per warp
+    bool at_once[2][3] = {{false}};        // whether all tiles are resident at once
     int *info = nullptr, *loc = nullptr, *cum = nullptr, *map = nullptr, *row = nullptr, *qgroup = nullptr;
     int64_t *gquad = nullptr;              // [groups] quads before each group
     unsigned char *s32 = nullptr, *s64 = nullptr;
@@ -110,6 +111,7 @@ struct DevLevel {
     TileDev tile[2][kTileParts];           // sweeps 0..7 and 7..0, each in tparts launches of 8 / tparts colours;
     int tparts = 0;                        // part q: colours from 8 q / tparts on (0: no plan)
     bool tfused = false;                   // a sweep 0..7 can form the residual in its launch, else tres does
+    bool tonce[2][3] = {{false}};          // so it is for all of the level's plans
     TileDev tres;
     // packed copy of A for the row kernels (packed.cu): per colour, 8-row groups of rows with
     // equal quad counts, entries quad-interleaved across the group; null pk_map when not built
@@ -267,7 +269,8 @@ struct Ctx {
     void *h_state = nullptr;          // pinned mirror: 64 bytes state + 16 doubles norms
     NarrowState narrow;               // shared-memory bottom of the V-cycle (narrow.cu)
     // the mixed solve's iterate as FP32 pairs for its outer residual (packed.cu)
-    float *xs_hi = nullptr, *xs_lo = nullptr;
+    float *xs_pair = nullptr;         // [n][2][R]
+    float4 *bs3 = nullptr;            // [n][R] and its right-hand side as three FP32 numbers
     // whole-sweep cooperative kernel (packed.cu): arrival counter and grid per lane count
     unsigned *sweep_bar = nullptr;
     int sweep_blocks[5] = {0, 0, 0, 0, 0};
@@ -339,18 +342,24 @@ void launch_packed_fill(const DevLevel &L, cudaStream_t s);
 // packed Gauss-Seidel colour / residual over rows [0, nrows); false when the level or the
 // matrix has no packed copy (the caller then uses the CSR kernels)
 template <class T> bool launch_packed_smooth(const DevLevel &L, int colour, const T *A, const T *dinv, const T *b,
-                                             T *x, int R, int tpb, cudaStream_t s, Chain *ch, int next = -1);
+                                             T *x, int R, int tpb, cudaStream_t s, Chain *ch, int next = -1,
+                                             int lim = INT32_MAX);
 template <class T> bool launch_packed_residual(const DevLevel &L, const T *A, const T *b, const T *x, T *r, int R,
                                                int nrows, int tpb, cudaStream_t s, Chain *ch);
 // r = b - A x at all rows of level L for the mixed solve's outer residual: x given as FP32 pairs
-// (xh + xl), the matrix as FP32 pairs, products and sums in pairs of FP32 (about 44 significant
+// (xp: [n][2][R], hi and lo parts of a row side by side), the matrix as FP32 pairs, products and sums in pairs of FP32 (about 44 significant
 // bits) and b - sum in FP64; false when the level has no packed copy
-bool launch_packed_residual_split(const DevLevel &L, const double *b, const float *xh, const float *xl, double *r,
-                                  int R, cudaStream_t s, Chain *ch);
-// xh, xl of an FP64 vector; x = xh + xl in FP64; x += e on the pair (FP32 two-sum)
-void launch_split(const double *x, float *xh, float *xl, int64_t n, cudaStream_t s);
-void launch_join(const float *xh, const float *xl, double *x, int64_t n, cudaStream_t s);
-void launch_add_pair(const float *e, float *xh, float *xl, int64_t n, cudaStream_t s, Chain *ch);
+bool launch_packed_residual_split(const DevLevel &L, const double *b, const float *xp, double *r, int R,
+                                  cudaStream_t s, Chain *ch);
+// the same at the end of a mixed iteration: b as three FP32 numbers (launch_split3), the result in FP32
+// (r32; z zeroed when given)
+bool launch_packed_outer(const DevLevel &L, const float4 *b3, const float *xp, float *r32, float *z, int R, int lanes,
+                         cudaStream_t s, Chain *ch);
+void launch_split3(const double *x, float4 *out, int64_t n, cudaStream_t s);
+// the pairs of an FP64 vector (xp may be x); x = hi + lo in FP64; x += e on the pairs (FP32 two-sum)
+void launch_split(const double *x, float *xp, int n, int R, cudaStream_t s);
+void launch_join(const float *xp, double *x, int n, int R, cudaStream_t s);
+void launch_add_pair(const float *e, float *xp, int n, int R, cudaStream_t s, Chain *ch);
 // a colour sequence (FP32) in one cooperative launch; bar: a device counter, status: the
 // bounded-wait word; false if the level has no packed copy or the launch is refused
 bool launch_packed_sweep(const DevLevel &L, const int *seq, int nseq, const float *dinv, const float *b, float *x,
@@ -383,7 +392,9 @@ template <class T> void launch_tile_sweep(const Ctx &c, const DevLevel &L, bool 
 // first sweep already done (1: the restriction applied colour 0's step from a zero start)
 template <class T> void launch_sweeps(const Ctx &c, const DevLevel &L, int sweeps, bool forward, const T *A,
                                       const T *dinv, const T *b, T *x, int R, cudaStream_t s, Chain *ch,
-                                      int skip = 0);
+                                      int skip = 0, bool from_zero = false);
+// whether launch_sweeps can take a zero start as given (from_zero) instead of reading zeros from x
+template <class T> bool sweeps_from_zero(const DevLevel &L);
 // next: the colour launched after this one on the same level (-1: none); its packed entries
 // are prefetched into L2 while this colour runs
 template <class T> void launch_smooth_colour(const DevLevel &L, int colour, const T *A, const T *dinv,
@@ -406,6 +417,7 @@ template <class T> void launch_coarse_apply(const Ctx &c, const DevLevel &L, con
 void launch_coarse_factor(const Ctx &c, const int *const *rps, const int *const *cis, const double *const *As,
                           cudaStream_t s);
 void launch_norms(const double *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch = nullptr);
+void launch_norms32(const float *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch = nullptr);
 // conjugate-gradient scalars in Ctx::pcg_s, four lanes each
 enum { kPcgRz = 0, kPcgS1 = 4, kPcgS2 = 8, kPcgAlpha = 12, kPcgBeta = 16, kPcgRz0 = 20, kPcgScalars = 24 };
 // a lane whose r.z has fallen below this fraction of its first value is converged to

@@ -72,17 +72,20 @@ __device__ __forceinline__ void load_row<double, 4>(const double *p, double (&v)
     v[0] = q0.x; v[1] = q0.y; v[2] = q1.x; v[3] = q1.y;
 }
 
+// kZero: a colour of the first sweep from a zero start; columns from lim on (the colour's first row) are
+// still zero and are left out without a look at x, so that x need not be zeroed and half the gathers fall
+// away.
 // One warp per group.  kGs: Gauss-Seidel update x += (b - A x) / A_ii (rows of one
 // colour, which never couple); otherwise r = b - A x.  Before the grid-dependency wait
 // a warp loads its group, its entries and (kGs) the inverse diagonal; after it, the
 // row's own b and x and the x gathers go out together.  x is read with plain loads: a
 // colour launch writes x only at rows of its own colour, which it never gathers.
-template <class T, int R, bool kGs>
+template <class T, int R, bool kGs, bool kZero>
 __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 *__restrict__ gq,
                                                      const int *__restrict__ rows, PkMat<T> m,
                                                      const T *__restrict__ dinv, const T *__restrict__ b, T *x,
                                                      T *__restrict__ r, const char *__restrict__ pf, int64_t pf_bytes,
-                                                     int pf_chunk, const PkRuns runs) {
+                                                     int pf_chunk, int lim, const PkRuns runs) {
     // the next colour's entries into L2 (static data, so before the grid-dependency wait):
     // one bulk prefetch of a 256-byte-aligned slice per block
     if (pf && threadIdx.x == 0) {
@@ -132,14 +135,19 @@ __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 
     T bv[R], xo[R];
     if (lead) {
         load_row<T, R>(b + (size_t)row * R, bv);
-        if (kGs) load_row<T, R>(x + (size_t)row * R, xo);
+        if (kGs && !kZero) load_row<T, R>(x + (size_t)row * R, xo);
+        if (kGs && kZero)
+#pragma unroll
+            for (int c = 0; c < R; c++) xo[c] = T(0);
     }
     T acc[R];
 #pragma unroll
     for (int c = 0; c < R; c++) acc[c] = T(0);
 #pragma unroll
     for (int q = 0; q < kPkPrefetch; q++) {
-        if (j[q] >= 0) {
+        // pads (-1) and, from a zero start, columns that are still zero; looked at only here, so that the
+        // entries stay in flight over the grid-dependency wait
+        if (kZero ? (unsigned)j[q] < (unsigned)lim : j[q] >= 0) {
             T xv[R];
             load_row<T, R>(x + (size_t)j[q] * R, xv);
 #pragma unroll
@@ -150,7 +158,7 @@ __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 
         int jj;
         T aa;
         m.get(base + 32 * q + lane, jj, aa);
-        if (jj >= 0) {
+        if (kZero ? (unsigned)jj < (unsigned)lim : jj >= 0) {
             T xv[R];
             load_row<T, R>(x + (size_t)jj * R, xv);
 #pragma unroll
@@ -201,16 +209,22 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// A vector of pairs keeps the hi and lo parts of a row side by side, [n][2][R]: a row of four components is
+// one 32-byte sector.  In two arrays its gather fetched two half-used sectors, and the residual was bound by
+// the sectors through L2 (72% busy) at 94 us on 927k rows.
 template <int R>
-__device__ __forceinline__ void ld_pair_row(const float *h, const float *l, float (&vh)[R], float (&vl)[R]) {
-#pragma unroll
-    for (int c = 0; c < R; c++) { vh[c] = h[c]; vl[c] = l[c]; }
-}
-template <>
-__device__ __forceinline__ void ld_pair_row<4>(const float *h, const float *l, float (&vh)[4], float (&vl)[4]) {
-    const float4 a = *reinterpret_cast<const float4 *>(h), b = *reinterpret_cast<const float4 *>(l);
-    vh[0] = a.x; vh[1] = a.y; vh[2] = a.z; vh[3] = a.w;
-    vl[0] = b.x; vl[1] = b.y; vl[2] = b.z; vl[3] = b.w;
+__device__ __forceinline__ void ld_pair_row(const float *p, float (&vh)[R], float (&vl)[R]) {
+    if constexpr (R == 4) {
+        const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+        vh[0] = a.x; vh[1] = a.y; vh[2] = a.z; vh[3] = a.w;
+        vl[0] = b.x; vl[1] = b.y; vl[2] = b.z; vl[3] = b.w;
+    } else if constexpr (R == 2) {
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        vh[0] = a.x; vh[1] = a.y; vl[0] = a.z; vl[1] = a.w;
+    } else {
+        const float2 a = *reinterpret_cast<const float2 *>(p);
+        vh[0] = a.x; vl[0] = a.y;
+    }
 }
 
 template <int R>
@@ -219,8 +233,7 @@ __global__ void __launch_bounds__(256) pk_split_residual_kernel(int g1, const in
                                                                 const int *__restrict__ col,
                                                                 const float2 *__restrict__ v2,
                                                                 const double *__restrict__ b,
-                                                                const float *__restrict__ xh,
-                                                                const float *__restrict__ xl,
+                                                                const float *__restrict__ xp,
                                                                 double *__restrict__ r) {
     const int lane = threadIdx.x & 31;
     const int g = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
@@ -247,7 +260,7 @@ __global__ void __launch_bounds__(256) pk_split_residual_kernel(int g1, const in
     for (int c = 0; c < R; c++) { sh[c] = 0.f; sl[c] = 0.f; }
     auto term = [&](int jj, float2 aa) {
         float vh[R], vl[R];
-        ld_pair_row<R>(xh + (size_t)jj * R, xl + (size_t)jj * R, vh, vl);
+        ld_pair_row<R>(xp + (size_t)jj * (2 * R), vh, vl);
 #pragma unroll
         for (int c = 0; c < R; c++) {
             const float p = __fmul_rn(aa.x, vh[c]);
@@ -287,35 +300,159 @@ __global__ void __launch_bounds__(256) pk_split_residual_kernel(int g1, const in
     }
 }
 
-// x += e on the FP32 pair (xh, xl): two-sum, then renormalise so that |xl| <= ulp(xh) / 2
-__global__ void add_pair_kernel(const float *__restrict__ e, float *__restrict__ xh, float *__restrict__ xl,
-                                int64_t n) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// The same residual at the end of a mixed V-cycle iteration: r rounded to FP32, the next cycle's right-hand
+// side (z, when given, zeroed as its start).  The right-hand side comes as three FP32 numbers (53 bits) and is
+// subtracted as pairs, so that no FP64 instruction is left (a warp issues one in about 64 cycles).  The norms
+// are a pass of their own over r32: summed here, the FP64 additions at every block's end held its place
+// (94 -> 140 us).  NC of the R components are live.
+template <int R, int NC>
+__global__ void __launch_bounds__(256) pk_outer_kernel(int g1, const int2 *__restrict__ gq, const int *__restrict__ rows,
+                                                       const int *__restrict__ col, const float2 *__restrict__ v2,
+                                                       const float4 *__restrict__ b3, const float *__restrict__ xp,
+                                                       float *__restrict__ r32, float *__restrict__ z) {
+    const int lane = threadIdx.x & 31, l = lane & 3;
+    const int g = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+    if (g >= g1) return;   // whole warps only
+    const int2 hd = __ldg(gq + g);
+    const int64_t base = (int64_t)(unsigned)hd.x * 32 + lane;
+    const int Q = hd.y;
+    const int row = __ldg(rows + 8 * (size_t)g + (lane >> 2));
+    int j[kPkPrefetch];
+    float2 a[kPkPrefetch];
+#pragma unroll
+    for (int q = 0; q < kPkPrefetch; q++) {
+        j[q] = -1;
+        a[q] = make_float2(0.f, 0.f);
+        if (q < Q) {
+            j[q] = __ldg(col + base + 32 * q);
+            a[q] = __ldg(v2 + base + 32 * q);
+        }
+    }
     grid_dep_wait();
     grid_dep_launch();
-    if (q >= n) return;
-    float s, err;
-    two_sum(xh[q], e[q], s, err);
-    const float t = __fadd_rn(xl[q], err);
-    const float h = __fadd_rn(s, t);                   // fast two-sum (|s| >= |t| after a two-sum)
-    xh[q] = h;
-    xl[q] = __fsub_rn(t, __fsub_rn(h, s));
+    float sh[R], sl[R];
+#pragma unroll
+    for (int c = 0; c < R; c++) { sh[c] = 0.f; sl[c] = 0.f; }
+    auto term = [&](int jj, float2 aa) {
+        float vh[R], vl[R];
+        ld_pair_row<R>(xp + (size_t)jj * (2 * R), vh, vl);
+#pragma unroll
+        for (int c = 0; c < NC; c++) {
+            const float p = __fmul_rn(aa.x, vh[c]);
+            const float t = fmaf(aa.x, vl[c], fmaf(aa.y, vh[c], fmaf(aa.x, vh[c], -p)));
+            float s2, e2;
+            two_sum(sh[c], p, s2, e2);
+            sh[c] = s2;
+            sl[c] += e2 + t;
+        }
+    };
+#pragma unroll
+    for (int q = 0; q < kPkPrefetch; q++)
+        if (j[q] >= 0) term(j[q], a[q]);
+    for (int q = kPkPrefetch; q < Q; q++) {   // rows of more than 32 entries
+        const int jj = __ldg(col + base + 32 * q);
+        if (jj >= 0) term(jj, __ldg(v2 + base + 32 * q));
+    }
+    // the four lanes' pairs are added so that lane c ends with component c
+    auto add_from = [&](float &h, float &lo, float gh, float gl, int o) {
+        float s2, e2;
+        two_sum(h, __shfl_xor_sync(kFull, gh, o, 4), s2, e2);
+        lo += __shfl_xor_sync(kFull, gl, o, 4) + e2;
+        h = s2;
+    };
+    float h, lo;
+    if constexpr (R == 4) {
+        const bool hi = l & 2, odd = l & 1;
+        float h0 = hi ? sh[2] : sh[0], l0 = hi ? sl[2] : sl[0], h1 = hi ? sh[3] : sh[1], l1 = hi ? sl[3] : sl[1];
+        add_from(h0, l0, hi ? sh[0] : sh[2], hi ? sl[0] : sl[2], 2);
+        add_from(h1, l1, hi ? sh[1] : sh[3], hi ? sl[1] : sl[3], 2);
+        h = odd ? h1 : h0; lo = odd ? l1 : l0;
+        add_from(h, lo, odd ? h0 : h1, odd ? l0 : l1, 1);
+    } else if constexpr (R == 2) {
+        const bool odd = l & 1;
+        h = odd ? sh[1] : sh[0]; lo = odd ? sl[1] : sl[0];
+        add_from(h, lo, odd ? sh[0] : sh[1], odd ? sl[0] : sl[1], 1);
+        add_from(h, lo, h, lo, 2);
+    } else {
+        h = sh[0]; lo = sl[0];
+        add_from(h, lo, h, lo, 1);
+        add_from(h, lo, h, lo, 2);
+    }
+    if (row >= 0 && l < R) {
+        const size_t q = (size_t)row * R + l;
+        float rr = 0.f;
+        if (l < NC) {
+            const float4 b = __ldg(b3 + q);
+            float s2, e2;
+            two_sum(b.x, -h, s2, e2);
+            rr = __fadd_rn(s2, __fadd_rn(__fadd_rn(e2, __fsub_rn(b.y, lo)), b.z));
+        }
+        r32[q] = rr;
+        if (z) z[q] = 0.f;
+    }
 }
 
-// x = xh + xl in FP64
-__global__ void join_kernel(const float *__restrict__ xh, const float *__restrict__ xl, double *__restrict__ x,
-                            int64_t n) {
+// x += e on the FP32 pairs: two-sum, then renormalise so that |lo| <= ulp(hi) / 2; one thread per row
+template <int R>
+__global__ void __launch_bounds__(256) add_pair_kernel(const float *__restrict__ e, float *xp, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dep_wait();
+    grid_dep_launch();
+    if (i >= n) return;
+    float ev[R], h[R], l[R];
+    load_row<float, R>(e + (size_t)i * R, ev);
+    float *p = xp + (size_t)i * (2 * R);
+    ld_pair_row<R>(p, h, l);
+#pragma unroll
+    for (int c = 0; c < R; c++) {
+        float s, err;
+        two_sum(h[c], ev[c], s, err);
+        const float t = __fadd_rn(l[c], err);
+        h[c] = __fadd_rn(s, t);                   // fast two-sum (|s| >= |t| after a two-sum)
+        l[c] = __fsub_rn(t, __fsub_rn(h[c], s));
+    }
+    if constexpr (R == 4) {
+        reinterpret_cast<float4 *>(p)[0] = make_float4(h[0], h[1], h[2], h[3]);
+        reinterpret_cast<float4 *>(p)[1] = make_float4(l[0], l[1], l[2], l[3]);
+    } else if constexpr (R == 2) {
+        *reinterpret_cast<float4 *>(p) = make_float4(h[0], h[1], l[0], l[1]);
+    } else {
+        *reinterpret_cast<float2 *>(p) = make_float2(h[0], l[0]);
+    }
+}
+
+// x = hi + lo in FP64
+__global__ void join_kernel(const float *__restrict__ xp, double *__restrict__ x, int64_t n, int R) {
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < n) x[q] = (double)xh[q] + (double)xl[q];
+    if (q >= n) return;
+    const float *p = xp + (q / R) * (2 * R) + q % R;
+    x[q] = (double)p[0] + (double)p[R];
 }
 
-__global__ void split_kernel(const double *__restrict__ x, float *__restrict__ xh, float *__restrict__ xl, int64_t n) {
+// x as three FP32 numbers, 53 bits, side by side (three arrays cost a gathered row three sectors)
+__global__ void split3_kernel(const double *__restrict__ x, float4 *__restrict__ out, int64_t n) {
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= n) return;
     const double v = x[q];
     const float h = (float)v;
-    xh[q] = h;
-    xl[q] = (float)(v - (double)h);
+    const double w = v - (double)h;
+    const float m = (float)w;
+    out[q] = make_float4(h, m, (float)(w - (double)m), 0.f);
+}
+
+// one thread per row, so that xp may be x itself
+template <int R>
+__global__ void split_kernel(const double *x, float *xp, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double v[R];
+    load_row<double, R>(x + (size_t)i * R, v);
+#pragma unroll
+    for (int c = 0; c < R; c++) {
+        const float h = (float)v[c];
+        xp[(size_t)i * (2 * R) + c] = h;
+        xp[(size_t)i * (2 * R) + R + c] = (float)(v[c] - (double)h);
+    }
 }
 
 template <class T> PkMat<T> pk_mat(const DevLevel &L);
@@ -330,7 +467,7 @@ template <> const double *level_A<double>(const DevLevel &L) { return L.A64; }
 template <class T, bool kGs>
 void launch_rows(const DevLevel &L, int g0, int g1, const T *dinv, const T *b, T *x, T *r, int R, int tpb,
                  cudaStream_t s, Chain *ch, const char *pf = nullptr, int64_t pf_bytes = 0,
-                 const PkRuns &runs = PkRuns()) {
+                 const PkRuns &runs = PkRuns(), int lim = INT32_MAX) {
     if (g1 <= g0) return;
     tpb = std::max(32, std::min(512, tpb / 32 * 32));
     const unsigned blocks = (unsigned)(((int64_t)(g1 - g0) * 32 + tpb - 1) / tpb);
@@ -342,9 +479,11 @@ void launch_rows(const DevLevel &L, int g0, int g1, const T *dinv, const T *b, T
     } else {
         pf = nullptr;
     }
-    auto k = R == 1 ? pk_row_kernel<T, 1, kGs> : R == 2 ? pk_row_kernel<T, 2, kGs> : pk_row_kernel<T, 4, kGs>;
+    auto k = R == 1 ? pk_row_kernel<T, 1, kGs, false> : R == 2 ? pk_row_kernel<T, 2, kGs, false> : pk_row_kernel<T, 4, kGs, false>;
+    if (kGs && lim != INT32_MAX)
+        k = R == 1 ? pk_row_kernel<T, 1, kGs, kGs> : R == 2 ? pk_row_kernel<T, 2, kGs, kGs> : pk_row_kernel<T, 4, kGs, kGs>;
     klaunch(k, blocks, (unsigned)tpb, 0, s, ch, g0, g1, (const int2 *)L.pk_gq, (const int *)L.pk_rows, pk_mat<T>(L),
-            dinv, b, x, r, pf, pf ? pf_bytes : (int64_t)0, chunk, runs);
+            dinv, b, x, r, pf, pf ? pf_bytes : (int64_t)0, chunk, lim, runs);
 }
 
 // ---- the finest level's whole sweep (all its colour steps) in one cooperative launch ----
@@ -573,33 +712,54 @@ void launch_packed_fill(const DevLevel &L, cudaStream_t s) {
                                                                         L.pk_e32, L.pk_v64, L.pk_v2);
 }
 
-bool launch_packed_residual_split(const DevLevel &L, const double *b, const float *xh, const float *xl, double *r,
-                                  int R, cudaStream_t s, Chain *ch) {
+bool launch_packed_residual_split(const DevLevel &L, const double *b, const float *xp, double *r, int R,
+                                  cudaStream_t s, Chain *ch) {
     if (!L.pk_map || !L.pk_v2) return false;
     const int g1 = L.pk_gs[9];
     if (g1 <= 0) return true;
     const unsigned blocks = (unsigned)(((int64_t)g1 * 32 + 255) / 256);
     auto k = R == 1 ? pk_split_residual_kernel<1> : R == 2 ? pk_split_residual_kernel<2> : pk_split_residual_kernel<4>;
     klaunch(k, blocks, 256u, 0, s, ch, g1, (const int2 *)L.pk_gq, (const int *)L.pk_rows, (const int *)L.pk_col,
-            (const float2 *)L.pk_v2, b, xh, xl, r);
+            (const float2 *)L.pk_v2, b, xp, r);
     return true;
 }
 
-void launch_add_pair(const float *e, float *xh, float *xl, int64_t n, cudaStream_t s, Chain *ch) {
-    if (n) klaunch(add_pair_kernel, (unsigned)((n + 255) / 256), 256u, 0, s, ch, e, xh, xl, n);
+void launch_add_pair(const float *e, float *xp, int n, int R, cudaStream_t s, Chain *ch) {
+    auto k = R == 1 ? add_pair_kernel<1> : R == 2 ? add_pair_kernel<2> : add_pair_kernel<4>;
+    if (n) klaunch(k, (unsigned)((n + 255) / 256), 256u, 0, s, ch, e, xp, n);
 }
 
-void launch_join(const float *xh, const float *xl, double *x, int64_t n, cudaStream_t s) {
-    if (n) join_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(xh, xl, x, n);
+void launch_join(const float *xp, double *x, int n, int R, cudaStream_t s) {
+    const int64_t m = (int64_t)n * R;
+    if (m) join_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(xp, x, m, R);
 }
 
-void launch_split(const double *x, float *xh, float *xl, int64_t n, cudaStream_t s) {
-    if (n) split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, xh, xl, n);
+bool launch_packed_outer(const DevLevel &L, const float4 *b3, const float *xp, float *r32, float *z, int R, int lanes,
+                         cudaStream_t s, Chain *ch) {
+    if (!L.pk_map || !L.pk_v2) return false;
+    auto k = R == 1 ? pk_outer_kernel<1, 1> : R == 2 ? pk_outer_kernel<2, 2>
+             : lanes == 3 ? pk_outer_kernel<4, 3> : pk_outer_kernel<4, 4>;
+    if (L.pk_gs[9] <= 0) return true;
+    klaunch(k, (unsigned)(((int64_t)L.pk_gs[9] * 32 + 255) / 256), 256u, 0, s, ch, L.pk_gs[9], (const int2 *)L.pk_gq, (const int *)L.pk_rows,
+            (const int *)L.pk_col, (const float2 *)L.pk_v2, b3, xp, r32, z);
+    return true;
+}
+
+void launch_split3(const double *x, float4 *out, int64_t n, cudaStream_t s) {
+    if (n) split3_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, out, n);
+}
+
+void launch_split(const double *x, float *xp, int n, int R, cudaStream_t s) {
+    if (n == 0) return;
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    if (R == 1) split_kernel<1><<<blocks, 256, 0, s>>>(x, xp, n);
+    else if (R == 2) split_kernel<2><<<blocks, 256, 0, s>>>(x, xp, n);
+    else split_kernel<4><<<blocks, 256, 0, s>>>(x, xp, n);
 }
 
 template <class T>
 bool launch_packed_smooth(const DevLevel &L, int colour, const T *A, const T *dinv, const T *b, T *x, int R, int tpb,
-                          cudaStream_t s, Chain *ch, int next) {
+                          cudaStream_t s, Chain *ch, int next, int lim) {
     if (!L.pk_map || A != level_A<T>(L)) return false;
     const char *pf = nullptr;
     int64_t pf_bytes = 0;
@@ -608,7 +768,7 @@ bool launch_packed_smooth(const DevLevel &L, int colour, const T *A, const T *di
         pf_bytes = (L.pk_es[next + 1] - L.pk_es[next]) * (int64_t)sizeof(int2);
     }
     launch_rows<T, true>(L, L.pk_gs[colour], L.pk_gs[colour + 1], dinv, b, x, nullptr, R, tpb, s, ch, pf, pf_bytes,
-                         L.pk_runs[colour]);
+                         L.pk_runs[colour], lim);
     return true;
 }
 
@@ -673,9 +833,9 @@ int packed_sweep_blocks(int R) {
 }
 
 template bool launch_packed_smooth<float>(const DevLevel &, int, const float *, const float *, const float *, float *,
-                                          int, int, cudaStream_t, Chain *, int);
+                                          int, int, cudaStream_t, Chain *, int, int);
 template bool launch_packed_smooth<double>(const DevLevel &, int, const double *, const double *, const double *,
-                                           double *, int, int, cudaStream_t, Chain *, int);
+                                           double *, int, int, cudaStream_t, Chain *, int, int);
 template bool launch_packed_residual<float>(const DevLevel &, const float *, const float *, const float *, float *,
                                             int, int, int, cudaStream_t, Chain *);
 template bool launch_packed_residual<double>(const DevLevel &, const double *, const double *, const double *,

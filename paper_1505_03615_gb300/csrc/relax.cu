@@ -215,7 +215,7 @@ ResidualFn<T> residual_fn(int tpr) {
 
 template <class T>
 void launch_sweeps(const Ctx &c, const DevLevel &L, int sweeps, bool forward, const T *A, const T *dinv, const T *b,
-                   T *x, int R, cudaStream_t s, Chain *ch, int skip) {
+                   T *x, int R, cudaStream_t s, Chain *ch, int skip, bool from_zero) {
     if (sweeps <= 0) return;
     skip = std::max(0, std::min(skip, 8));
     const LaunchShape &sh = L.shape[sizeof(T) == 8][kShapeSmooth];
@@ -235,8 +235,20 @@ void launch_sweeps(const Ctx &c, const DevLevel &L, int sweeps, bool forward, co
             // the colour that follows on this level: the next of this sweep, or the first of the next sweep
             const int nq = q < 7 ? q + 1 : (sw + 1 < sweeps ? 0 : -1);
             const int next = nq < 0 ? -1 : (forward ? nq : 7 - nq);
-            launch_smooth_colour<T>(L, colour, A, dinv, b, x, R, s, ch, next);
+            if (from_zero && sw == 0 && forward) {
+                const int tpb = sh.tpb;
+                if (L.cs[colour + 1] > L.cs[colour])
+                    launch_packed_smooth<T>(L, colour, A, dinv, b, x, R, tpb, s, ch, next, L.cs[colour]);
+            } else {
+                launch_smooth_colour<T>(L, colour, A, dinv, b, x, R, s, ch, next);
+            }
         }
+}
+
+template <class T>
+bool sweeps_from_zero(const DevLevel &L) {
+    const LaunchShape &sh = L.shape[sizeof(T) == 8][kShapeSmooth];
+    return L.pk_map && sh.tpr == 4 && sh.tpb != kSweepShapeTpb;
 }
 
 template <class T>
@@ -567,8 +579,8 @@ __device__ __forceinline__ double block_sum(const double (&acc)[R]) {
 
 // One round of blocks over the GPU, a row's components in one or two vector loads.  (256 blocks and scalar
 // loads took 38 us for 927k rows of four components, 30 MB.)
-template <int R>
-__global__ void __launch_bounds__(256) norm_partial_kernel(const double *__restrict__ v, int n, double *__restrict__ part) {
+template <class T, int R>
+__global__ void __launch_bounds__(256) norm_partial_kernel(const T *__restrict__ v, int n, double *__restrict__ part) {
     grid_dep_wait();
     grid_dep_launch();
     double acc[R];
@@ -576,10 +588,10 @@ __global__ void __launch_bounds__(256) norm_partial_kernel(const double *__restr
     for (int r = 0; r < R; r++) acc[r] = 0.0;
 #pragma unroll 4
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double x[R];
-        load_x<double, R>(v + (size_t)i * R, x);
+        T x[R];
+        load_x<T, R>(v + (size_t)i * R, x);
 #pragma unroll
-        for (int r = 0; r < R; r++) acc[r] = fma(x[r], x[r], acc[r]);
+        for (int r = 0; r < R; r++) acc[r] = fma((double)x[r], (double)x[r], acc[r]);
     }
     const double t = block_sum<R>(acc);
     if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = t;
@@ -799,7 +811,12 @@ void launch_pcg_update(double *x, double *r, const double *p, const double *q, c
 }
 
 void launch_norms(const double *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch) {
-    auto k = R == 1 ? norm_partial_kernel<1> : R == 2 ? norm_partial_kernel<2> : norm_partial_kernel<4>;
+    auto k = R == 1 ? norm_partial_kernel<double, 1> : R == 2 ? norm_partial_kernel<double, 2> : norm_partial_kernel<double, 4>;
+    klaunch(k, (unsigned)kNormBlocks, 256u, 0, s, ch, v, n, part);
+    klaunch(norm_final_kernel, 1u, 128u, 0, s, ch, (const double *)part, (int)kNormBlocks, R, out);
+}
+void launch_norms32(const float *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch) {
+    auto k = R == 1 ? norm_partial_kernel<float, 1> : R == 2 ? norm_partial_kernel<float, 2> : norm_partial_kernel<float, 4>;
     klaunch(k, (unsigned)kNormBlocks, 256u, 0, s, ch, v, n, part);
     klaunch(norm_final_kernel, 1u, 128u, 0, s, ch, (const double *)part, (int)kNormBlocks, R, out);
 }
@@ -866,7 +883,8 @@ void launch_add_double(double *x, const double *e, int64_t n, cudaStream_t s) {
 // explicit instantiations
 #define LBMG_INST(T)                                                                                           \
     template void launch_sweeps<T>(const Ctx &, const DevLevel &, int, bool, const T *, const T *, const T *, T *, \
-                                   int, cudaStream_t, Chain *, int);                                          \
+                                   int, cudaStream_t, Chain *, int, bool);                                    \
+    template bool sweeps_from_zero<T>(const DevLevel &);                                                       \
     template void launch_smooth_colour<T>(const DevLevel &, int, const T *, const T *, const T *, T *, int,   \
                                           cudaStream_t, Chain *, int);                                         \
     template void launch_residual<T>(const DevLevel &, const T *, const T *, const T *, T *, int, cudaStream_t, int, \

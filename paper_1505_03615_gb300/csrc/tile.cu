@@ -12,9 +12,12 @@
 // cycles of the 200k-triangle knot at depth 8 went from 394 to 285 us mixed and from 1225 to 840 us FP64.
 //
 // Where the line lies (kTileLevel32, kTileLevel64): the rim costs work, about 3.5 times the own entries at
-// 64 rows a tile, 1.5 to 2 at 500 rows in two launches per sweep of four colours each.  Measured per FP32
-// sweep of torus-knot levels, colour launches / tiles: 18 / 6 us at 5,000 rows, 18 / 10 at 78,000, 28 / 27
-// at 232,000, 76 / 71-79 at 927,000; FP64 at three right-hand sides 42 / 14, 42 / 37, 60 / 70, 290 / 310.
+// 64 rows a tile, 1.5 to 2 at 250 rows in two launches per sweep of four colours each, and every plan has a
+// copy of the entries, which on larger levels pushes the other levels' data out of L2.  Measured per FP32
+// sweep of torus-knot levels, colour launches / tiles: 18 / 5.5 us at 5,000 rows, 18 / 7.5 at 19,000, 18 / 11
+// at 78,000, 28 / 27 at 232,000, 76 / 71-79 at 927,000; a cycle of the 1M-triangle sheets with four
+// components took 1410 us with 91,000 rows tiled, 1283 without.  FP64 at three right-hand sides: 42 / 14 us,
+// 42 / 30, 42 / 37, 60 / 70, 290 / 310.
 //
 // Four lanes share a row, as in packed.cu, so that a row's gathers are few per lane and all in flight
 // together (a step is one chain of shared-memory latencies); the lanes' sums are added so that lane c ends
@@ -431,7 +434,7 @@ constexpr int kTileStatic = 3072;   // upper bound of the kernel's static shared
 // level, so a tile is fetched whole where that leaves room for the blocks the launch has per SM; on large
 // levels three or two blocks share an SM, each with at least two groups per warp on their way.
 template <class T>
-int tile_ring(const TileDev &t, int R, int sms, int sm_bytes, int block_bytes) {
+int tile_ring(const TileDev &t, int R, int sms, int sm_bytes, int block_bytes, bool &at_once) {
     const int whole = std::min(kTileRing, (t.maxgrp + kTileWarps - 1) / kTileWarps);
     auto fits = [&](int ring, int blocks) {
         const size_t need = tile_smem<T>(t, R, ring);
@@ -440,7 +443,7 @@ int tile_ring(const TileDev &t, int R, int sms, int sm_bytes, int block_bytes) {
     const int want = std::max(1, std::min(3, (t.ntile + sms - 1) / sms));
     for (int blocks = want; blocks >= 1; blocks--)
         for (int ring = whole; ring >= (blocks == 1 ? 1 : std::min(whole, 2)); ring--)
-            if (fits(ring, blocks)) return ring;
+            if (fits(ring, blocks)) { at_once = blocks == want; return ring; }
     return 0;
 }
 
@@ -486,8 +489,8 @@ bool tile_fits(const TilePlan &p, TileDev &t) {
     if (!smem_limits(l)) { cudaGetLastError(); return false; }
     const int rs[3] = {1, 2, 4};
     for (int q = 0; q < 3; q++) {
-        t.ring[0][q] = tile_ring<float>(t, rs[q], l.sms, l.sm, l.block);
-        t.ring[1][q] = tile_ring<double>(t, rs[q], l.sms, l.sm, l.block);
+        t.ring[0][q] = tile_ring<float>(t, rs[q], l.sms, l.sm, l.block, t.at_once[0][q]);
+        t.ring[1][q] = tile_ring<double>(t, rs[q], l.sms, l.sm, l.block, t.at_once[1][q]);
         if (t.ring[0][q] < 1 || t.ring[1][q] < 1) return false;
     }
     return true;

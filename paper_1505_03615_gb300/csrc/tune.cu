@@ -67,7 +67,7 @@ cudaError_t time_kernel(Ctx &c, DevLevel &L, int kind, int R, int reps, cudaEven
     ch.on = c.pdl != 0;   // the capture stream is an ordinary stream
     TileVec<T> tv{V<T>::x(L), V<T>::y(L)};
     for (int q = 0; q < reps; q++) {
-        if (kind == kShapeSmooth && L.tparts > 0 && L.shape[sizeof(T) == 8][kind].tile) {
+        if (kind == kShapeSmooth && L.tparts > 0 && L.tonce[sizeof(T) == 8][R >> 1] && L.shape[sizeof(T) == 8][kind].tile) {
             launch_tile_sweep<T>(c, L, true, tv, V<T>::b(L), (T *)nullptr, R, cs, &ch);
         } else if (kind == kShapeSmooth) {
             launch_sweeps<T>(c, L, 1, true, V<T>::A(L), V<T>::dinv(L), V<T>::b(L), V<T>::x(L), R, cs, &ch);
@@ -163,7 +163,7 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
                 }
             }
             // the tiled sweep, kept unless a shape above is faster (it saves the cycle launches besides)
-            if (kind == kShapeSmooth && L.tparts > 0) {
+            if (kind == kShapeSmooth && L.tparts > 0 && L.tonce[fp64][R >> 1]) {
                 LaunchShape tl;
                 L.shape[fp64][kind] = tl;
                 float ms = 0.f;
