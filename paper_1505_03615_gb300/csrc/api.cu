@@ -269,7 +269,7 @@ void enqueue_smooth(Ctx &c, DevLevel &L, int R, int sweeps, bool forward, cudaSt
         }
     } else if (c.smoother == LBMG_JACOBI) {
         for (int sw = 0; sw < sweeps; sw++) {
-            launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch);
+            launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch, c.lanes);
             launch_jacobi_update<T>(L, P<T>::dinv(L), P<T>::r(L), P<T>::x(L), (T)c.omega, R, s);
             if (ch) ch->cut();
         }
@@ -339,7 +339,7 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
         } else {
             enqueue_smooth<T>(c, L, R, c.nu1, true, s, ch, skip, d == top && zero_start && top_from_zero<T>(c, d, R));
             if (timed && d == top) record(c.ev_smooth[1], s, ch);
-            launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch);
+            launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch, c.lanes);
         }
         // the shared-memory bottom starts level dn from zero itself; the dense solve overwrites d0
         // (and a tiled level's first sweep starts from zero without reading it)
@@ -404,7 +404,7 @@ void enqueue_cycle_level(Ctx &c, int d, int R, cudaStream_t s, Chain *ch) {
     }
     DevLevel &Lc = c.lev[d - 1];
     enqueue_smooth<T>(c, L, R, c.nu1, true, s, ch);
-    launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch);
+    launch_residual<T>(L, P<T>::A(L), P<T>::b(L), P<T>::x(L), P<T>::r(L), R, s, L.ns, ch, c.lanes);
     launch_restrict<T>(Lc, P<T>::r(L), P<T>::b(Lc), R, s, P<T>::x(Lc), ch);
     for (int g = 0; g < c.gamma; g++) enqueue_cycle_level<T>(c, d - 1, R, s, ch);
     launch_prolong_add<T>(L, P<T>::x(Lc), P<T>::x(L), R, s, ch);
@@ -482,7 +482,7 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
         launch_add_double(c.xs, F.x64, m, s);
         ch.cut();
     }
-    launch_residual<double>(F, F.A64, c.bs, c.xs, c.rs, R, s, -1, &ch);
+    launch_residual<double>(F, F.A64, c.bs, c.xs, c.rs, R, s, -1, &ch, c.lanes);
     launch_norms(c.rs, F.n, R, c.norm_part, c.norm_out, s, &ch);
 }
 
@@ -493,7 +493,7 @@ void enqueue_pcg_product(Ctx &c, DevLevel &F, int R, int precision, int64_t m, c
         launch_split(c.pcg_p, c.xs_pair, F.n, R, s);
         if (launch_packed_residual_split(F, c.pcg_zero, c.xs_pair, c.pcg_q, R, s, nullptr)) return;
     }
-    launch_residual<double>(F, F.A64, c.pcg_zero, c.pcg_p, c.pcg_q, R, s);
+    launch_residual<double>(F, F.A64, c.pcg_zero, c.pcg_p, c.pcg_q, R, s, -1, nullptr, c.lanes);
 }
 
 // one step of conjugate gradients preconditioned by the V-cycle, in the flexible
@@ -1393,7 +1393,7 @@ static int solve_cond(lbmg_handle h, cudaGraphExec_t exec, const double *rd, con
     LBMG_CK(cudaEventRecord(c.ev0, s));
     launch_pack(rd, Fl.n, nrhs, R, c.bs, s, c.fperm);
     launch_pack(xin, Fl.n, nrhs, R, c.xs, s, c.fperm);
-    launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s);
+    launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s, -1, nullptr, c.lanes);
     const size_t m = (size_t)Fl.n * R;
     const bool pairs = pair_iterate(c, precision, pcg);
     if (pairs) enqueue_pair_start(c, R, s);
@@ -1469,7 +1469,7 @@ static int solve_pcg_batch(lbmg_handle h, const double *rd, const double *xin, d
     LBMG_CK(cudaEventRecord(c.ev0, s));
     launch_pack(rd, Fl.n, nrhs, R, c.bs, s, c.fperm);
     launch_pack(xin, Fl.n, nrhs, R, c.xs, s, c.fperm);
-    launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s);
+    launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s, -1, nullptr, c.lanes);
     const size_t m = (size_t)Fl.n * R;
     LBMG_CK(cudaMemsetAsync(c.pcg_z, 0, m * sizeof(double), s));
     LBMG_CK(cudaMemsetAsync(c.pcg_p, 0, m * sizeof(double), s));
@@ -1639,7 +1639,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
     LBMG_CK(cudaEventRecord(c.ev0, s));
     launch_pack(rd, Fl.n, nrhs, R, c.bs, s, c.fperm);
     launch_pack(xin, Fl.n, nrhs, R, c.xs, s, c.fperm);
-    launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s);
+    launch_residual<double>(Fl, Fl.A64, c.bs, c.xs, c.rs, R, s, -1, nullptr, c.lanes);
     const bool pairs = pair_iterate(c, precision, pcg);
     if (pairs) enqueue_pair_start(c, R, s);
     if (pcg) {
@@ -1811,7 +1811,7 @@ int lbmg_residual(lbmg_handle h, int d, const double *rhs, const double *x, doub
     launch_pack(bd, L.n, nrhs, R, L.b64, s);
     LBMG_TRY(input_ptr(h, x, cnt, 1, s, &xd));
     launch_pack(xd, L.n, nrhs, R, L.x64, s);
-    launch_residual<double>(L, L.A64, L.b64, L.x64, L.r64, R, s);
+    launch_residual<double>(L, L.A64, L.b64, L.x64, L.r64, R, s, -1, nullptr, nrhs);
     LBMG_TRY(output_ptr(h, r, cnt, 0, &rd, &host_out));
     launch_unpack(L.r64, L.n, nrhs, R, rd, s);
     return finish_output(r, rd, cnt, host_out, s);

@@ -339,13 +339,14 @@ bool packed_layout(const HostLevel &hl, std::vector<int32_t> &gq, std::vector<in
                    std::vector<int32_t> &map, std::vector<int32_t> &col, int gs[10], int64_t *total);
 // refresh the packed FP32 and FP64 values from the level's CSR A32 / A64 (after assembly)
 void launch_packed_fill(const DevLevel &L, cudaStream_t s);
+// (lanes: live right-hand sides, 3 leaves out the padding of three to four)
 // packed Gauss-Seidel colour / residual over rows [0, nrows); false when the level or the
 // matrix has no packed copy (the caller then uses the CSR kernels)
 template <class T> bool launch_packed_smooth(const DevLevel &L, int colour, const T *A, const T *dinv, const T *b,
                                              T *x, int R, int tpb, cudaStream_t s, Chain *ch, int next = -1,
-                                             int lim = INT32_MAX);
+                                             int lim = INT32_MAX, int lanes = 0);
 template <class T> bool launch_packed_residual(const DevLevel &L, const T *A, const T *b, const T *x, T *r, int R,
-                                               int nrows, int tpb, cudaStream_t s, Chain *ch);
+                                               int nrows, int tpb, cudaStream_t s, Chain *ch, int lanes = 0);
 // r = b - A x at all rows of level L for the mixed solve's outer residual: x given as FP32 pairs
 // (xp: [n][2][R], hi and lo parts of a row side by side), the matrix as FP32 pairs, products and sums in pairs of FP32 (about 44 significant
 // bits) and b - sum in FP64; false when the level has no packed copy
@@ -399,9 +400,9 @@ template <class T> bool sweeps_from_zero(const DevLevel &L);
 // are prefetched into L2 while this colour runs
 template <class T> void launch_smooth_colour(const DevLevel &L, int colour, const T *A, const T *dinv,
                                              const T *b, T *x, int R, cudaStream_t s, Chain *ch = nullptr,
-                                             int next = -1);
+                                             int next = -1, int lanes = 0);
 template <class T> void launch_residual(const DevLevel &L, const T *A, const T *b, const T *x, T *r, int R,
-                                        cudaStream_t s, int nrows = -1, Chain *ch = nullptr);
+                                        cudaStream_t s, int nrows = -1, Chain *ch = nullptr, int lanes = 0);
 template <class T> void launch_jacobi_update(const DevLevel &L, const T *dinv, const T *r, T *x, T omega, int R,
                                              cudaStream_t s);
 // bc = P^T rf; when xc is given, the coarse correction xc is zeroed in the same pass, or, with

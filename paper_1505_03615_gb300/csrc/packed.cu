@@ -75,12 +75,16 @@ __device__ __forceinline__ void load_row<double, 4>(const double *p, double (&v)
 // kZero: a colour of the first sweep from a zero start; columns from lim on (the colour's first row) are
 // still zero and are left out without a look at x, so that x need not be zeroed and half the gathers fall
 // away.
+// NC of the R components are live (three right-hand sides padded to four); each is summed, updated and written
+// by a lane of its own.  GB300's FP64 pipe takes a warp instruction in 64 cycles or so, and the FP64 kernels are
+// bound by their number: eight rows of 18 entries take 20 for three right-hand sides, where four components
+// summed by every lane and updated by one took 36 (an FP64 sweep of 927k rows: 388 -> 250 us).
 // One warp per group.  kGs: Gauss-Seidel update x += (b - A x) / A_ii (rows of one
 // colour, which never couple); otherwise r = b - A x.  Before the grid-dependency wait
 // a warp loads its group, its entries and (kGs) the inverse diagonal; after it, the
 // row's own b and x and the x gathers go out together.  x is read with plain loads: a
 // colour launch writes x only at rows of its own colour, which it never gathers.
-template <class T, int R, bool kGs, bool kZero>
+template <class T, int R, int NC, bool kGs, bool kZero>
 __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 *__restrict__ gq,
                                                      const int *__restrict__ rows, PkMat<T> m,
                                                      const T *__restrict__ dinv, const T *__restrict__ b, T *x,
@@ -119,7 +123,8 @@ __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 
         Q = hd.y;
     }
     const int row = __ldg(rows + 8 * (size_t)g + (lane >> 2));
-    const bool lead = row >= 0 && (lane & 3) == 0;
+    const int l = lane & 3;
+    const bool mine = row >= 0;
     int j[kPkPrefetch];
     T a[kPkPrefetch];
 #pragma unroll
@@ -129,16 +134,15 @@ __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 
         if (q < Q) m.get(base + 32 * q + lane, j[q], a[q]);
     }
     T d = T(0);
-    if (kGs && lead) d = __ldg(dinv + row);
+    if (kGs && mine) d = __ldg(dinv + row);
     grid_dep_wait();
     grid_dep_launch();
-    T bv[R], xo[R];
-    if (lead) {
-        load_row<T, R>(b + (size_t)row * R, bv);
-        if (kGs && !kZero) load_row<T, R>(x + (size_t)row * R, xo);
-        if (kGs && kZero)
-#pragma unroll
-            for (int c = 0; c < R; c++) xo[c] = T(0);
+    // lane l < NC of a row ends with component l
+    const size_t at = (size_t)(mine ? row : 0) * R + l;
+    T bv = T(0), xo = T(0);
+    if (mine && l < NC) {
+        bv = b[at];
+        if (kGs && !kZero) xo = x[at];
     }
     T acc[R];
 #pragma unroll
@@ -151,7 +155,7 @@ __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 
             T xv[R];
             load_row<T, R>(x + (size_t)j[q] * R, xv);
 #pragma unroll
-            for (int c = 0; c < R; c++) acc[c] = fma(a[q], xv[c], acc[c]);
+            for (int c = 0; c < NC; c++) acc[c] = fma(a[q], xv[c], acc[c]);
         }
     }
     for (int q = kPkPrefetch; q < Q; q++) {   // rows of more than 32 entries
@@ -162,20 +166,35 @@ __global__ void __launch_bounds__(512) pk_row_kernel(int g0, int g1, const int2 
             T xv[R];
             load_row<T, R>(x + (size_t)jj * R, xv);
 #pragma unroll
-            for (int c = 0; c < R; c++) acc[c] = fma(aa, xv[c], acc[c]);
+            for (int c = 0; c < NC; c++) acc[c] = fma(aa, xv[c], acc[c]);
         }
     }
-#pragma unroll
-    for (int o = 2; o > 0; o >>= 1)
-#pragma unroll
-        for (int c = 0; c < R; c++) acc[c] += __shfl_xor_sync(kFull, acc[c], o, 4);
-    if (lead) {
+    // the lanes' sums, lanes l and l ^ 2 first, halved so that lane l keeps component l
+    T sum;
+    if constexpr (R == 4) {
+        const bool hi = l & 2, odd = l & 1;
+        T k0 = hi ? acc[2] : acc[0], k1 = hi ? acc[3] : acc[1];
+        const T g0s = hi ? acc[0] : acc[2], g1s = hi ? acc[1] : acc[3];
+        k0 += __shfl_xor_sync(kFull, g0s, 2);
+        k1 += __shfl_xor_sync(kFull, g1s, 2);
+        const T give = odd ? k0 : k1;
+        sum = (odd ? k1 : k0) + __shfl_xor_sync(kFull, give, 1);
+    } else if constexpr (R == 2) {
+        const T k0 = acc[0] + __shfl_xor_sync(kFull, acc[0], 2), k1 = acc[1] + __shfl_xor_sync(kFull, acc[1], 2);
+        const bool odd = l & 1;
+        const T give = odd ? k0 : k1;
+        sum = (odd ? k1 : k0) + __shfl_xor_sync(kFull, give, 1);
+    } else {
+        sum = acc[0] + __shfl_xor_sync(kFull, acc[0], 2);
+        sum += __shfl_xor_sync(kFull, sum, 1);
+    }
+    if (mine && l < R) {
+        const T v = kGs ? xo + (bv - sum) * d : bv - sum;
         if (kGs) {
-#pragma unroll
-            for (int c = 0; c < R; c++) x[(size_t)row * R + c] = xo[c] + (bv[c] - acc[c]) * d;
+            if (l < NC) x[at] = v;
+            else if (kZero) x[at] = T(0);   // the pad
         } else {
-#pragma unroll
-            for (int c = 0; c < R; c++) r[(size_t)row * R + c] = bv[c] - acc[c];
+            r[at] = l < NC ? v : T(0);
         }
     }
 }
@@ -465,7 +484,7 @@ template <> const double *level_A<double>(const DevLevel &L) { return L.A64; }
 // pf, pf_bytes: a byte range to prefetch into L2 (null: none), split over the blocks in
 // 256-byte-aligned slices
 template <class T, bool kGs>
-void launch_rows(const DevLevel &L, int g0, int g1, const T *dinv, const T *b, T *x, T *r, int R, int tpb,
+void launch_rows(const DevLevel &L, int g0, int g1, const T *dinv, const T *b, T *x, T *r, int R, int lanes, int tpb,
                  cudaStream_t s, Chain *ch, const char *pf = nullptr, int64_t pf_bytes = 0,
                  const PkRuns &runs = PkRuns(), int lim = INT32_MAX) {
     if (g1 <= g0) return;
@@ -479,9 +498,13 @@ void launch_rows(const DevLevel &L, int g0, int g1, const T *dinv, const T *b, T
     } else {
         pf = nullptr;
     }
-    auto k = R == 1 ? pk_row_kernel<T, 1, kGs, false> : R == 2 ? pk_row_kernel<T, 2, kGs, false> : pk_row_kernel<T, 4, kGs, false>;
+    auto k = R == 1   ? pk_row_kernel<T, 1, 1, kGs, false>
+             : R == 2 ? pk_row_kernel<T, 2, 2, kGs, false>
+             : lanes == 3 ? pk_row_kernel<T, 4, 3, kGs, false> : pk_row_kernel<T, 4, 4, kGs, false>;
     if (kGs && lim != INT32_MAX)
-        k = R == 1 ? pk_row_kernel<T, 1, kGs, kGs> : R == 2 ? pk_row_kernel<T, 2, kGs, kGs> : pk_row_kernel<T, 4, kGs, kGs>;
+        k = R == 1   ? pk_row_kernel<T, 1, 1, kGs, kGs>
+            : R == 2 ? pk_row_kernel<T, 2, 2, kGs, kGs>
+            : lanes == 3 ? pk_row_kernel<T, 4, 3, kGs, kGs> : pk_row_kernel<T, 4, 4, kGs, kGs>;
     klaunch(k, blocks, (unsigned)tpb, 0, s, ch, g0, g1, (const int2 *)L.pk_gq, (const int *)L.pk_rows, pk_mat<T>(L),
             dinv, b, x, r, pf, pf ? pf_bytes : (int64_t)0, chunk, lim, runs);
 }
@@ -759,7 +782,7 @@ void launch_split(const double *x, float *xp, int n, int R, cudaStream_t s) {
 
 template <class T>
 bool launch_packed_smooth(const DevLevel &L, int colour, const T *A, const T *dinv, const T *b, T *x, int R, int tpb,
-                          cudaStream_t s, Chain *ch, int next, int lim) {
+                          cudaStream_t s, Chain *ch, int next, int lim, int lanes) {
     if (!L.pk_map || A != level_A<T>(L)) return false;
     const char *pf = nullptr;
     int64_t pf_bytes = 0;
@@ -767,21 +790,21 @@ bool launch_packed_smooth(const DevLevel &L, int colour, const T *A, const T *di
         pf = reinterpret_cast<const char *>(L.pk_e32 + L.pk_es[next]);
         pf_bytes = (L.pk_es[next + 1] - L.pk_es[next]) * (int64_t)sizeof(int2);
     }
-    launch_rows<T, true>(L, L.pk_gs[colour], L.pk_gs[colour + 1], dinv, b, x, nullptr, R, tpb, s, ch, pf, pf_bytes,
+    launch_rows<T, true>(L, L.pk_gs[colour], L.pk_gs[colour + 1], dinv, b, x, nullptr, R, lanes, tpb, s, ch, pf, pf_bytes,
                          L.pk_runs[colour], lim);
     return true;
 }
 
 template <class T>
 bool launch_packed_residual(const DevLevel &L, const T *A, const T *b, const T *x, T *r, int R, int nrows, int tpb,
-                            cudaStream_t s, Chain *ch) {
+                            cudaStream_t s, Chain *ch, int lanes) {
     if (!L.pk_map || A != level_A<T>(L)) return false;
     // the group ranges end exactly at the smoothed rows (ns) and at all rows (n)
     int g1;
     if (nrows == L.n) g1 = L.pk_gs[9];
     else if (nrows == L.ns) g1 = L.pk_gs[8];
     else return false;
-    launch_rows<T, false>(L, 0, g1, (const T *)nullptr, b, const_cast<T *>(x), r, R, tpb, s, ch);
+    launch_rows<T, false>(L, 0, g1, (const T *)nullptr, b, const_cast<T *>(x), r, R, lanes, tpb, s, ch);
     return true;
 }
 
@@ -833,12 +856,12 @@ int packed_sweep_blocks(int R) {
 }
 
 template bool launch_packed_smooth<float>(const DevLevel &, int, const float *, const float *, const float *, float *,
-                                          int, int, cudaStream_t, Chain *, int, int);
+                                          int, int, cudaStream_t, Chain *, int, int, int);
 template bool launch_packed_smooth<double>(const DevLevel &, int, const double *, const double *, const double *,
-                                           double *, int, int, cudaStream_t, Chain *, int, int);
+                                           double *, int, int, cudaStream_t, Chain *, int, int, int);
 template bool launch_packed_residual<float>(const DevLevel &, const float *, const float *, const float *, float *,
-                                            int, int, int, cudaStream_t, Chain *);
+                                            int, int, int, cudaStream_t, Chain *, int);
 template bool launch_packed_residual<double>(const DevLevel &, const double *, const double *, const double *,
-                                             double *, int, int, int, cudaStream_t, Chain *);
+                                             double *, int, int, int, cudaStream_t, Chain *, int);
 
 }  // namespace lbmg

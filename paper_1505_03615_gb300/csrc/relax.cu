@@ -238,9 +238,9 @@ void launch_sweeps(const Ctx &c, const DevLevel &L, int sweeps, bool forward, co
             if (from_zero && sw == 0 && forward) {
                 const int tpb = sh.tpb;
                 if (L.cs[colour + 1] > L.cs[colour])
-                    launch_packed_smooth<T>(L, colour, A, dinv, b, x, R, tpb, s, ch, next, L.cs[colour]);
+                    launch_packed_smooth<T>(L, colour, A, dinv, b, x, R, tpb, s, ch, next, L.cs[colour], c.lanes);
             } else {
-                launch_smooth_colour<T>(L, colour, A, dinv, b, x, R, s, ch, next);
+                launch_smooth_colour<T>(L, colour, A, dinv, b, x, R, s, ch, next, c.lanes);
             }
         }
 }
@@ -253,13 +253,13 @@ bool sweeps_from_zero(const DevLevel &L) {
 
 template <class T>
 void launch_smooth_colour(const DevLevel &L, int colour, const T *A, const T *dinv, const T *b, T *x, int R,
-                          cudaStream_t s, Chain *ch, int next) {
+                          cudaStream_t s, Chain *ch, int next, int lanes) {
     const int r0 = L.cs[colour], r1 = L.cs[colour + 1];
     if (r1 <= r0) return;
     const LaunchShape &sh = L.shape[sizeof(T) == 8][kShapeSmooth];
     // four threads per row: the packed copy of the matrix (one 256-byte load per warp and quad)
     const int tpb = sh.tpb == kSweepShapeTpb ? 256 : sh.tpb;   // one colour of a whole-sweep level
-    if (sh.tpr == 4 && launch_packed_smooth<T>(L, colour, A, dinv, b, x, R, tpb, s, ch, next)) return;
+    if (sh.tpr == 4 && launch_packed_smooth<T>(L, colour, A, dinv, b, x, R, tpb, s, ch, next, INT32_MAX, lanes)) return;
     const unsigned blocks = (unsigned)(((int64_t)(r1 - r0) * sh.tpr + tpb - 1) / tpb);
     const SmoothFn<T> k = R == 1 ? smooth_fn<T, 1>(sh.tpr) : R == 2 ? smooth_fn<T, 2>(sh.tpr) : smooth_fn<T, 4>(sh.tpr);
     klaunch(k, blocks, (unsigned)tpb, 0, s, ch, r0, r1, L.rp, L.ci, A, dinv, b, x);
@@ -267,11 +267,11 @@ void launch_smooth_colour(const DevLevel &L, int colour, const T *A, const T *di
 
 template <class T>
 void launch_residual(const DevLevel &L, const T *A, const T *b, const T *x, T *r, int R, cudaStream_t s, int nrows,
-                     Chain *ch) {
+                     Chain *ch, int lanes) {
     const int n = nrows < 0 ? L.n : nrows;
     if (n == 0) return;
     const LaunchShape &sh = L.shape[sizeof(T) == 8][kShapeResidual];
-    if (sh.tpr == 4 && launch_packed_residual<T>(L, A, b, x, r, R, n, sh.tpb, s, ch)) return;
+    if (sh.tpr == 4 && launch_packed_residual<T>(L, A, b, x, r, R, n, sh.tpb, s, ch, lanes)) return;
     const unsigned blocks = (unsigned)(((int64_t)n * sh.tpr + sh.tpb - 1) / sh.tpb);
     const ResidualFn<T> k =
         R == 1 ? residual_fn<T, 1>(sh.tpr) : R == 2 ? residual_fn<T, 2>(sh.tpr) : residual_fn<T, 4>(sh.tpr);
@@ -886,9 +886,9 @@ void launch_add_double(double *x, const double *e, int64_t n, cudaStream_t s) {
                                    int, cudaStream_t, Chain *, int, bool);                                    \
     template bool sweeps_from_zero<T>(const DevLevel &);                                                       \
     template void launch_smooth_colour<T>(const DevLevel &, int, const T *, const T *, const T *, T *, int,   \
-                                          cudaStream_t, Chain *, int);                                         \
+                                          cudaStream_t, Chain *, int, int);                                    \
     template void launch_residual<T>(const DevLevel &, const T *, const T *, const T *, T *, int, cudaStream_t, int, \
-                                     Chain *);                                                                 \
+                                     Chain *, int);                                                            \
     template void launch_jacobi_update<T>(const DevLevel &, const T *, const T *, T *, T, int, cudaStream_t);   \
     template void launch_restrict<T>(const DevLevel &, const T *, T *, int, cudaStream_t, T *, Chain *, bool); \
     template void launch_prolong_add<T>(const DevLevel &, const T *, T *, int, cudaStream_t, Chain *);         \
