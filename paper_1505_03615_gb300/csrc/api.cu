@@ -1333,12 +1333,11 @@ int lbmg_assemble(lbmg_handle h, double t, void *stream) {
     if (!h || !(t >= 0) || !std::isfinite(t)) return LBMG_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     Ctx &c = h->c;
-    if (!c.moments_ready) {   // build-time geometry: once per hierarchy
-        launch_fragment_moments(c, s);
-        c.moments_ready = true;
-    }
-    launch_fine_gather(c, t, s);
-    for (int d = c.D - 1; d >= c.d0; d--) launch_galerkin(c, d, t, s);
+    const bool first = !c.moments_ready;   // build-time geometry: once per hierarchy
+    if (first) launch_fragment_moments(c, s);
+    launch_fine_gather(c, t, first, s);
+    for (int d = c.D - 1; d >= c.d0; d--) launch_galerkin(c, d, t, first, s);
+    c.moments_ready = true;
     for (int d = c.d0; d <= c.D; d++) launch_inverse_diag(c.lev[d], c.diag_part, s);
     for (int d = c.d0 + 1; d <= c.D; d++) launch_packed_fill(c.lev[d], s);
     for (int d = c.d0 + 1; d <= c.D; d++) launch_tile_fill(c.lev[d], s);

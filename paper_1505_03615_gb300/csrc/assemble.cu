@@ -235,92 +235,128 @@ void launch_fragment_moments(const Ctx &c, cudaStream_t s) {
                                                            c.moments, c.stage);
 }
 
+// ---- sums over contribution lists: kGatherLanes lanes share a stored entry ----
+// Neighbouring lanes read neighbouring list entries and every lane's values are four in flight; one thread per
+// entry read the lists an entry apart (each 32-byte sector for 4 bytes at a time) and took 14 ms for the coarse
+// levels of the 927k-row knots.  The stiffness depends on the build-time geometry alone, as the pieces'
+// integrals do: it is summed by the first assembly (kL) and only read by later ones, which halves the gathers.
+constexpr int kGatherLanes = 8;
+
+// sum over the kGatherLanes lanes of an entry, in all of them
+__device__ __forceinline__ double lanes_sum(double v) {
+#pragma unroll
+    for (int o = kGatherLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__device__ __forceinline__ void store_entry(int64_t s, double m, double l, double t, bool with_l, double *M, double *L,
+                                            double *A64, float *A32) {
+    M[s] = m;
+    if (with_l) L[s] = l;
+    const double a = m + t * l;
+    A64[s] = a;
+    A32[s] = (float)a;
+}
+
 // finest level: sum the local-pair contributions of every stored entry
-__global__ void fine_gather_kernel(int64_t nnz, const int64_t *__restrict__ arp, const uint32_t *__restrict__ aidx,
-                                   const double2 *__restrict__ stage, const double *__restrict__ fscale, double t,
-                                   double *__restrict__ M, double *__restrict__ L, double *__restrict__ A64,
-                                   float *__restrict__ A32) {
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= nnz) return;
+template <bool kL>
+__global__ void __launch_bounds__(256) fine_gather_kernel(int64_t nnz, const int64_t *__restrict__ arp,
+                                                          const uint32_t *__restrict__ aidx,
+                                                          const double2 *__restrict__ stage,
+                                                          const double *__restrict__ fscale, double t,
+                                                          double *__restrict__ M, double *__restrict__ L,
+                                                          double *__restrict__ A64, float *__restrict__ A32) {
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t s = tid / kGatherLanes;
+    const int lane = (int)(tid % kGatherLanes);
+    const bool active = s < nnz;
     double m = 0.0, l = 0.0;
-    const int64_t k1 = arp[s + 1];
-    int64_t k = arp[s];
-    // eight list entries, then their eight values, in flight together; the sum keeps its order
-    for (; k + 8 <= k1; k += 8) {
-        uint32_t ix[8];
+    const int64_t k1 = active ? __ldg(arp + s + 1) : 0;
+    for (int64_t k = active ? __ldg(arp + s) + lane : 0; k < k1; k += 4 * kGatherLanes) {
+        uint32_t ix[4];
 #pragma unroll
-        for (int u = 0; u < 8; u++) ix[u] = __ldg(aidx + k + u);
-        double2 v[8];
-        double w[8];
+        for (int u = 0; u < 4; u++) ix[u] = k + u * kGatherLanes < k1 ? __ldg(aidx + k + u * kGatherLanes) : 0u;
+        double vm[4], vl[4], w[4];
 #pragma unroll
-        for (int u = 0; u < 8; u++) { v[u] = __ldg(stage + ix[u]); w[u] = __ldg(fscale + ix[u] / kStagePerFrag); }
-#pragma unroll
-        for (int u = 0; u < 8; u++) { m = fma(v[u].x, w[u], m); l += v[u].y; }
-    }
-    for (; k < k1; k++) {
-        const uint32_t ix = aidx[k];
-        const double2 v = __ldg(stage + ix);
-        m = fma(v.x, __ldg(fscale + ix / kStagePerFrag), m);
-        l += v.y;
-    }
-    M[s] = m;
-    L[s] = l;
-    const double a = m + t * l;
-    A64[s] = a;
-    A32[s] = (float)a;
-}
-
-void launch_fine_gather(const Ctx &c, double t, cudaStream_t s) {
-    const DevLevel &L = c.lev[c.D];
-    const int threads = 256;
-    fine_gather_kernel<<<(unsigned)((L.nnz + threads - 1) / threads), threads, 0, s>>>(
-        L.nnz, c.arp, c.aidx, reinterpret_cast<const double2 *>(c.stage), c.frag_scale, t, L.M, L.L, L.A64, L.A32);
-}
-
-// coarse level: (P^T A P)_ab = sum over listed fine entries of 2^-e A_il
-__global__ void galerkin_kernel(int64_t nnz, const int64_t *__restrict__ grp, const uint32_t *__restrict__ gidx,
-                                const double *__restrict__ Mf, const double *__restrict__ Lf, double t,
-                                double *__restrict__ M, double *__restrict__ L, double *__restrict__ A64,
-                                float *__restrict__ A32) {
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= nnz) return;
-    double m = 0.0, l = 0.0;
-    const int64_t k1 = grp[s + 1];
-    int64_t k = grp[s];
-    // eight list entries, then their sixteen values, in flight together; the sum keeps its order
-    for (; k + 8 <= k1; k += 8) {
-        uint32_t e[8];
-#pragma unroll
-        for (int u = 0; u < 8; u++) e[u] = __ldg(gidx + k + u);
-        double mv[8], lv[8];
-#pragma unroll
-        for (int u = 0; u < 8; u++) { mv[u] = __ldg(Mf + (e[u] & kGalMask)); lv[u] = __ldg(Lf + (e[u] & kGalMask)); }
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const double w = ldexp(1.0, -(int)(e[u] >> kGalShift));
-            m = fma(w, mv[u], m);
-            l = fma(w, lv[u], l);
+        for (int u = 0; u < 4; u++) {
+            vm[u] = vl[u] = w[u] = 0.0;
+            if (k + u * kGatherLanes < k1) {
+                if (kL) {
+                    const double2 v = __ldg(stage + ix[u]);
+                    vm[u] = v.x; vl[u] = v.y;
+                } else {
+                    vm[u] = __ldg(&stage[ix[u]].x);
+                }
+                w[u] = __ldg(fscale + ix[u] / kStagePerFrag);
+            }
         }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (k + u * kGatherLanes < k1) {
+                m = fma(vm[u], w[u], m);
+                if (kL) l += vl[u];
+            }
     }
-    for (; k < k1; k++) {
-        const uint32_t e = __ldg(gidx + k);
-        const uint32_t idx = e & kGalMask;
-        const double w = ldexp(1.0, -(int)(e >> kGalShift));
-        m = fma(w, __ldg(Mf + idx), m);
-        l = fma(w, __ldg(Lf + idx), l);
-    }
-    M[s] = m;
-    L[s] = l;
-    const double a = m + t * l;
-    A64[s] = a;
-    A32[s] = (float)a;
+    m = lanes_sum(m);
+    if (kL) l = lanes_sum(l);
+    if (active && lane == 0) store_entry(s, m, kL ? l : L[s], t, kL, M, L, A64, A32);
 }
 
-void launch_galerkin(const Ctx &c, int dc, double t, cudaStream_t s) {
+void launch_fine_gather(const Ctx &c, double t, bool with_l, cudaStream_t s) {
+    const DevLevel &L = c.lev[c.D];
+    if (L.nnz == 0) return;
+    const unsigned blocks = (unsigned)((L.nnz * kGatherLanes + 255) / 256);
+    auto k = with_l ? fine_gather_kernel<true> : fine_gather_kernel<false>;
+    k<<<blocks, 256, 0, s>>>(L.nnz, c.arp, c.aidx, reinterpret_cast<const double2 *>(c.stage), c.frag_scale, t, L.M,
+                             L.L, L.A64, L.A32);
+}
+
+// coarse level: (P^T A P)_ab = sum over listed fine entries of 2^-e A_il (the weight from its exponent bits: a
+// call of ldexp cost more instructions than the rest)
+template <bool kL>
+__global__ void __launch_bounds__(256) galerkin_kernel(int64_t nnz, const int64_t *__restrict__ grp,
+                                                       const uint32_t *__restrict__ gidx, const double *__restrict__ Mf,
+                                                       const double *__restrict__ Lf, double t, double *__restrict__ M,
+                                                       double *__restrict__ L, double *__restrict__ A64,
+                                                       float *__restrict__ A32) {
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t s = tid / kGatherLanes;
+    const int lane = (int)(tid % kGatherLanes);
+    const bool active = s < nnz;
+    double m = 0.0, l = 0.0;
+    const int64_t k1 = active ? __ldg(grp + s + 1) : 0;
+    for (int64_t k = active ? __ldg(grp + s) + lane : 0; k < k1; k += 4 * kGatherLanes) {
+        uint32_t e[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) e[u] = k + u * kGatherLanes < k1 ? __ldg(gidx + k + u * kGatherLanes) : 0u;
+        double mv[4], lv[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            mv[u] = lv[u] = 0.0;
+            if (k + u * kGatherLanes < k1) {
+                mv[u] = __ldg(Mf + (e[u] & kGalMask));
+                if (kL) lv[u] = __ldg(Lf + (e[u] & kGalMask));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (k + u * kGatherLanes < k1) {
+                const double w = __hiloint2double((1023 - (int)(e[u] >> kGalShift)) << 20, 0);
+                m = fma(w, mv[u], m);
+                if (kL) l = fma(w, lv[u], l);
+            }
+    }
+    m = lanes_sum(m);
+    if (kL) l = lanes_sum(l);
+    if (active && lane == 0) store_entry(s, m, kL ? l : L[s], t, kL, M, L, A64, A32);
+}
+
+void launch_galerkin(const Ctx &c, int dc, double t, bool with_l, cudaStream_t s) {
     const DevLevel &Lc = c.lev[dc], &Lf = c.lev[dc + 1];
-    const int threads = 256;
-    galerkin_kernel<<<(unsigned)((Lc.nnz + threads - 1) / threads), threads, 0, s>>>(
-        Lc.nnz, Lc.grp, Lc.gidx, Lf.M, Lf.L, t, Lc.M, Lc.L, Lc.A64, Lc.A32);
+    if (Lc.nnz == 0) return;
+    const unsigned blocks = (unsigned)((Lc.nnz * kGatherLanes + 255) / 256);
+    auto k = with_l ? galerkin_kernel<true> : galerkin_kernel<false>;
+    k<<<blocks, 256, 0, s>>>(Lc.nnz, Lc.grp, Lc.gidx, Lf.M, Lf.L, t, Lc.M, Lc.L, Lc.A64, Lc.A32);
 }
 
 // Relaxation skips rows whose diagonal is below this fraction of the level's mean

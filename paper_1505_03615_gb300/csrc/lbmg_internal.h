@@ -183,7 +183,7 @@ struct Ctx {
     double *frag_scale = nullptr;          // [nfrag] physical area per finest-unit area
     // the pieces' moments and local (M, L) integrals in finest-unit area depend only on the
     // build-time geometry: computed by the first assembly, reused by the next (frag_scale enters
-    // in fine_gather_kernel)
+    // in fine_gather_kernel), and with them the stiffness matrices of all levels
     bool moments_ready = false;
     int *fperm = nullptr;                  // [nu] user finest index -> finest row
     int *fiperm = nullptr;                 // [n_D] finest row -> user index
@@ -324,8 +324,9 @@ int lobpcg(Ctx &c, int k, double tol, int max_iters, const double *X_user, doubl
 
 // ----- kernels (assemble.cu) -----
 void launch_fragment_moments(const Ctx &c, cudaStream_t s);
-void launch_fine_gather(const Ctx &c, double t, cudaStream_t s);
-void launch_galerkin(const Ctx &c, int dc, double t, cudaStream_t s);
+// with_l: sum the stiffness too (the first assembly; it depends on the build-time geometry alone)
+void launch_fine_gather(const Ctx &c, double t, bool with_l, cudaStream_t s);
+void launch_galerkin(const Ctx &c, int dc, double t, bool with_l, cudaStream_t s);
 // FP64 and FP32 inverse diagonals, 0 for rows below 1e-20 of the level's mean diagonal;
 // part: 256 doubles of scratch (per-block sums of the diagonal)
 void launch_inverse_diag(const DevLevel &L, double *part, cudaStream_t s);
