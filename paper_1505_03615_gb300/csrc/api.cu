@@ -486,70 +486,53 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
     launch_norms(c.rs, F.n, R, c.norm_part, c.norm_out, s, &ch);
 }
 
-// q = -A p of a CG step: in mixed precision with p's FP64 values carried as FP32 pairs
-// (the product of the outer residual), else in FP64
-void enqueue_pcg_product(Ctx &c, DevLevel &F, int R, int precision, int64_t m, cudaStream_t s) {
-    if (precision == LBMG_MIXED && F.pk_v2) {
-        launch_split(c.pcg_p, c.xs_pair, F.n, R, s);
-        if (launch_packed_residual_split(F, c.pcg_zero, c.xs_pair, c.pcg_q, R, s, nullptr)) return;
-    }
-    launch_residual<double>(F, F.A64, c.pcg_zero, c.pcg_p, c.pcg_q, R, s, -1, nullptr, c.lanes);
+// what a CG iteration finds prepared: the residual as the cycle's right-hand side
+void enqueue_pcg_start(Ctx &c, int R, int precision, cudaStream_t s) {
+    DevLevel &F = c.lev[c.D];
+    const int64_t m = (int64_t)F.n * R;
+    if (precision == LBMG_MIXED) launch_to_float(c.rs, F.b32, m, s);
+    else cudaMemcpyAsync(F.b64, c.rs, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
+}
+
+PcgRows pcg_rows(const Ctx &c) {
+    if (c.ninst > 1) return {c.ditem, c.ditem_start, c.row_inst, c.nditem, c.ninst, c.lev[c.D].n};
+    return {nullptr, nullptr, nullptr, 0, 1, c.lev[c.D].n};
 }
 
 // one step of conjugate gradients preconditioned by the V-cycle, in the flexible
-// (Polak-Ribiere) form, each right-hand side lane with its own step lengths:
-//   s2 = r.z_old;  z = Vcycle(r);  s1 = r.z;  beta = (s1 - s2) / rz;  rz = s1;
+// (Polak-Ribiere) form, each right-hand side lane (of each mesh of a batch) with its own step lengths:
+//   z = Vcycle(r);  s2 = r.z_old;  s1 = r.z;  beta = (s1 - s2) / rz;  rz = s1;
 //   p = z + beta p;  q = -A p;  alpha = s1 / (p.A p);  x += alpha p;  r -= alpha A p;  norms(r)
-void enqueue_pcg_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed = true) {
+// q in mixed precision with p's FP64 values carried as FP32 pairs (the product of the outer residual)
+template <class T>
+void enqueue_pcg_step(Ctx &c, int R, bool timed, cudaStream_t s) {
     DevLevel &F = c.lev[c.D];
     const int64_t m = (int64_t)F.n * R;
-    launch_pcg_dot(c.rs, c.pcg_z, F.n, R, c.pcg_part, c.pcg_s, 0, s);
+    const bool batch = c.ninst > 1;
+    const PcgRows w = pcg_rows(c);
+    double *sc = batch ? c.pcg_si : c.pcg_s;
+    const double *norms = batch ? c.inst_norm : nullptr, *tol = batch ? c.pcg_tol : nullptr;
     Chain ch = make_chain(c, s);
-    if (precision == LBMG_MIXED) {
-        launch_to_float(c.rs, F.b32, m, s, top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32, &ch);
-        enqueue_cycle<float>(c, R, s, timed, &ch);
-        to_double_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(F.x32, c.pcg_z, m);
-    } else {
-        cudaMemcpyAsync(F.b64, c.rs, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
-        if (!top_from_zero<double>(c, c.D, R)) cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
-        enqueue_cycle<double>(c, R, s, timed, &ch);
-        cudaMemcpyAsync(c.pcg_z, F.x64, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    }
-    launch_pcg_dot(c.rs, c.pcg_z, F.n, R, c.pcg_part, c.pcg_s, 1, s);
-    launch_pcg_direction(c.pcg_z, c.pcg_p, c.pcg_s, F.n, R, s);
-    enqueue_pcg_product(c, F, R, precision, m, s);
-    launch_pcg_dot(c.pcg_p, c.pcg_q, F.n, R, c.pcg_part, c.pcg_s, 2, s);
-    launch_pcg_update(c.xs, c.rs, c.pcg_p, c.pcg_q, c.pcg_s, F.n, R, s);
-    launch_norms(c.rs, F.n, R, c.norm_part, c.norm_out, s);
+    if (!top_from_zero<T>(c, c.D, R)) cudaMemsetAsync(P<T>::x(F), 0, m * sizeof(T), s);
+    if (batch) enqueue_vcycle<T>(c, R, s, false, &ch);
+    else enqueue_cycle<T>(c, R, s, timed, &ch);
+    launch_pcg_z<T>(w, c.rs, P<T>::x(F), c.pcg_z, R, c.pcg_part, s, &ch);
+    launch_pcg_scalar(w, R, c.pcg_part, sc, 1, norms, tol, s, &ch);
+    const bool pairs = sizeof(T) == 4 && F.pk_v2;
+    launch_pcg_direction(w, c.pcg_z, c.pcg_p, sc, pairs ? c.xs_pair : nullptr, R, s, &ch);
+    if (!pairs || !launch_packed_residual_split(F, c.pcg_zero, c.xs_pair, c.pcg_q, R, s, &ch))
+        launch_residual<double>(F, F.A64, c.pcg_zero, c.pcg_p, c.pcg_q, R, s, -1, &ch, c.lanes);
+    launch_pcg_dot(w, c.pcg_p, c.pcg_q, nullptr, nullptr, R, c.pcg_part, s, &ch);
+    launch_pcg_scalar(w, R, c.pcg_part, sc, 2, norms, tol, s, &ch);
+    launch_pcg_update<T>(w, c.xs, c.rs, c.pcg_p, c.pcg_q, sc, P<T>::b(F), R, c.pcg_part, s, &ch);
+    // (||b||^2 of a batch's meshes stays from the start of the solve)
+    if (batch) launch_pcg_sum(w, c.pcg_part, c.inst_norm, 16, 4, R, s, &ch);
+    else launch_pcg_sum(w, c.pcg_part, c.norm_out, 0, 4, R, s, &ch);
 }
 
-// the same step for a batch: every mesh has its own step lengths (per-mesh dot products
-// over the finest-level work items), and the per-mesh norms of r and b end the step
-void enqueue_pcg_batch_iteration(Ctx &c, int R, int precision, cudaStream_t s) {
-    DevLevel &F = c.lev[c.D];
-    const int64_t m = (int64_t)F.n * R;
-    launch_item_dot2(c.nitem, c.nnitem, c.rs, c.pcg_z, nullptr, nullptr, R, c.item_part, s);
-    launch_inst_pcg_scalar(c.item_start, c.ninst, R, c.item_part, c.pcg_si, 0, c.inst_norm, c.pcg_tol, s);
-    Chain ch = make_chain(c, s);
-    if (precision == LBMG_MIXED) {
-        launch_to_float(c.rs, F.b32, m, s, top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32, &ch);
-        enqueue_vcycle<float>(c, R, s, false, &ch);
-        to_double_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(F.x32, c.pcg_z, m);
-    } else {
-        cudaMemcpyAsync(F.b64, c.rs, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
-        if (!top_from_zero<double>(c, c.D, R)) cudaMemsetAsync(F.x64, 0, m * sizeof(double), s);
-        enqueue_vcycle<double>(c, R, s, false, &ch);
-        cudaMemcpyAsync(c.pcg_z, F.x64, m * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    }
-    launch_item_dot2(c.nitem, c.nnitem, c.rs, c.pcg_z, nullptr, nullptr, R, c.item_part, s);
-    launch_inst_pcg_scalar(c.item_start, c.ninst, R, c.item_part, c.pcg_si, 1, c.inst_norm, c.pcg_tol, s);
-    launch_inst_pcg_direction(c.pcg_z, c.pcg_p, c.pcg_si, c.row_inst, F.n, R, s);
-    enqueue_pcg_product(c, F, R, precision, m, s);
-    launch_item_dot2(c.nitem, c.nnitem, c.pcg_p, c.pcg_q, nullptr, nullptr, R, c.item_part, s);
-    launch_inst_pcg_scalar(c.item_start, c.ninst, R, c.item_part, c.pcg_si, 2, c.inst_norm, c.pcg_tol, s);
-    launch_inst_pcg_update(c.xs, c.rs, c.pcg_p, c.pcg_q, c.pcg_si, c.row_inst, F.n, R, s);
-    launch_item_dot2(c.nitem, c.nnitem, c.rs, c.rs, c.bs, c.bs, R, c.item_part, s);
-    launch_inst_sum(c.item_start, c.ninst, c.item_part, c.inst_norm, 16, s);
+void enqueue_pcg_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed = true) {
+    if (precision == LBMG_MIXED) enqueue_pcg_step<float>(c, R, timed, s);
+    else enqueue_pcg_step<double>(c, R, timed, s);
 }
 
 int get_graph(lbmg_handle h, int R, int precision, bool pcg, cudaGraphExec_t *out) {
@@ -562,8 +545,7 @@ int get_graph(lbmg_handle h, int R, int precision, bool pcg, cudaGraphExec_t *ou
     }
     if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }
     LBMG_CK(cudaStreamBeginCapture(c.capture_stream, cudaStreamCaptureModeThreadLocal));
-    if (pcg && c.ninst > 1) enqueue_pcg_batch_iteration(c, R, precision, c.capture_stream);
-    else if (pcg) enqueue_pcg_iteration(c, R, precision, c.capture_stream);
+    if (pcg) enqueue_pcg_iteration(c, R, precision, c.capture_stream);
     else enqueue_iteration(c, R, precision, c.capture_stream);
     cudaGraph_t graph = nullptr;
     LBMG_CK(cudaStreamEndCapture(c.capture_stream, &graph));
@@ -625,8 +607,7 @@ int build_cond_graph(Ctx &c, int R, int precision, bool pcg, cudaGraphExec_t *ou
     LBMG_CK(cudaGraphAddNode(&loop, g, &begin, nullptr, 1, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     LBMG_CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    if (pcg && batch) enqueue_pcg_batch_iteration(c, R, precision, cs);
-    else if (pcg) enqueue_pcg_iteration(c, R, precision, cs, false);
+    if (pcg) enqueue_pcg_iteration(c, R, precision, cs, false);
     else enqueue_iteration(c, R, precision, cs, false);
     ctl_step_kernel<<<1, 32, 0, cs>>>(c.ctl, c.norm_out, batch ? c.inst_norm : nullptr, c.ninst, c.narrow.status,
                                       c.flag, hc);
@@ -899,11 +880,18 @@ int upload_hierarchy(lbmg_handle h) {
     c.nnitem = (int)(c.nitem_host.size() / 3);
     LBMG_TRY(h->upload(&c.nitem, c.nitem_host));
     {
-        // the items are generated mesh by mesh: mesh m owns items [start[m], start[m + 1])
-        std::vector<int32_t> start(c.ninst + 1, 0);
-        for (int it = 0; it < c.nnitem; it++) start[c.nitem_host[3 * it] + 1]++;
-        for (int m = 0; m < c.ninst; m++) start[m + 1] += start[m];
-        LBMG_TRY(h->upload(&c.item_start, start));
+        // the smaller items of the batch CG's sums, generated mesh by mesh: mesh m owns [start[m], start[m + 1])
+        std::vector<int32_t> item, start(c.ninst + 1, 0);
+        for (int m = 0; m < c.ninst; m++) {
+            for (int q = 0; q < 8; q++) {
+                const int s0 = H.seg[2 * (8 * m + q)], s1 = H.seg[2 * (8 * m + q) + 1];
+                for (int r = s0; r < s1; r += kDotRows) item.insert(item.end(), {m, r, std::min(s1, r + kDotRows)});
+            }
+            start[m + 1] = (int32_t)(item.size() / 3);
+        }
+        c.nditem = (int)(item.size() / 3);
+        LBMG_TRY(h->upload(&c.ditem, item));
+        LBMG_TRY(h->upload(&c.ditem_start, start));
         LBMG_TRY(h->upload(&c.row_inst, H.lev[H.D].inst));
         LBMG_TRY(h->alloc(&c.pcg_si, (size_t)kPcgScalars * c.ninst));
         LBMG_TRY(h->alloc(&c.pcg_tol, 1));
@@ -938,7 +926,7 @@ int upload_hierarchy(lbmg_handle h) {
     LBMG_TRY(h->alloc(&c.pcg_zero, 4 * nD));
     LBMG_CK(cudaMemset(c.pcg_zero, 0, 4 * nD * sizeof(double)));
     LBMG_TRY(h->alloc(&c.pcg_s, (size_t)kPcgScalars));
-    LBMG_TRY(h->alloc(&c.pcg_part, 4 * (size_t)kNormBlocks));
+    LBMG_TRY(h->alloc(&c.pcg_part, 8 * (size_t)std::max(kNormBlocks, c.nditem)));
     LBMG_TRY(h->alloc(&c.diag_part, 256));
     LBMG_TRY(h->alloc(&c.norm_out, 8));
     LBMG_CK(cudaMemset(c.norm_out, 0, 8 * sizeof(double)));
@@ -1397,6 +1385,7 @@ static int solve_cond(lbmg_handle h, cudaGraphExec_t exec, const double *rd, con
     const bool pairs = pair_iterate(c, precision, pcg);
     if (pairs) enqueue_pair_start(c, R, s);
     if (pcg) {
+        enqueue_pcg_start(c, R, precision, s);
         LBMG_CK(cudaMemsetAsync(c.pcg_z, 0, m * sizeof(double), s));
         LBMG_CK(cudaMemsetAsync(c.pcg_p, 0, m * sizeof(double), s));
         if (batch) LBMG_CK(cudaMemsetAsync(c.pcg_si, 0, sizeof(double) * kPcgScalars * c.ninst, s));
@@ -1405,8 +1394,8 @@ static int solve_cond(lbmg_handle h, cudaGraphExec_t exec, const double *rd, con
     ctl_setup_kernel<<<1, 32, 0, s>>>(c.ctl, check ? tol : 0.0, max_cycles, check ? 0 : 1, nrhs,
                                       batch ? c.pcg_tol : nullptr);
     if (batch) {
-        launch_item_dot2(c.nitem, c.nnitem, c.rs, c.rs, c.bs, c.bs, R, c.item_part, s);
-        launch_inst_sum(c.item_start, c.ninst, c.item_part, c.inst_norm, 16, s);
+        launch_pcg_dot(pcg_rows(c), c.rs, c.rs, c.bs, c.bs, R, c.pcg_part, s, nullptr);
+        launch_pcg_sum(pcg_rows(c), c.pcg_part, c.inst_norm, 16, 8, R, s, nullptr);
     } else {
         launch_norms(c.bs, Fl.n, R, c.norm_part, c.norm_b, s);
         launch_norms(c.rs, Fl.n, R, c.norm_part, c.norm_out, s);
@@ -1475,8 +1464,9 @@ static int solve_pcg_batch(lbmg_handle h, const double *rd, const double *xin, d
     LBMG_CK(cudaMemsetAsync(c.pcg_si, 0, sizeof(double) * kPcgScalars * c.ninst, s));
     h->pcg_tol_host = tol;
     LBMG_CK(cudaMemcpyAsync(c.pcg_tol, &h->pcg_tol_host, sizeof(double), cudaMemcpyHostToDevice, s));
-    launch_item_dot2(c.nitem, c.nnitem, c.rs, c.rs, c.bs, c.bs, R, c.item_part, s);
-    launch_inst_sum(c.item_start, c.ninst, c.item_part, c.inst_norm, 16, s);
+    enqueue_pcg_start(c, R, precision, s);
+    launch_pcg_dot(pcg_rows(c), c.rs, c.rs, c.bs, c.bs, R, c.pcg_part, s, nullptr);
+    launch_pcg_sum(pcg_rows(c), c.pcg_part, c.inst_norm, 16, 8, R, s, nullptr);
     std::vector<double> &nh = h->inst_norm_host;
     nh.assign(16 * (size_t)c.ninst, 0.0);
     h->syncs = 0;
@@ -1510,7 +1500,7 @@ static int solve_pcg_batch(lbmg_handle h, const double *rd, const double *xin, d
         if (bad) { status = LBMG_DIVERGED; break; }
         if (conv || it >= max_iters) break;
         if (exec) LBMG_CK(cudaGraphLaunch(exec, s));
-        else enqueue_pcg_batch_iteration(c, R, precision, s);
+        else enqueue_pcg_iteration(c, R, precision, s, false);
         LBMG_TRY(read());
         it++;
     }
@@ -1642,6 +1632,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
     const bool pairs = pair_iterate(c, precision, pcg);
     if (pairs) enqueue_pair_start(c, R, s);
     if (pcg) {
+        enqueue_pcg_start(c, R, precision, s);
         LBMG_CK(cudaMemsetAsync(c.pcg_z, 0, (size_t)Fl.n * R * sizeof(double), s));
         LBMG_CK(cudaMemsetAsync(c.pcg_p, 0, (size_t)Fl.n * R * sizeof(double), s));
         LBMG_CK(cudaMemsetAsync(c.pcg_s, 0, kPcgScalars * sizeof(double), s));

@@ -232,7 +232,8 @@ struct Ctx {
     // batches: per-mesh scalars [ninst][kPcgScalars], the first work item of each mesh, finest row -> mesh
     double *pcg_si = nullptr;
     double *pcg_tol = nullptr;     // [1] tolerance of the running batch solve
-    int *item_start = nullptr, *row_inst = nullptr;
+    int *ditem = nullptr, *ditem_start = nullptr, *row_inst = nullptr;   // work items of kDotRows rows
+    int nditem = 0;
     double *h_norm = nullptr;    // pinned [8]
     SolveCtl *ctl = nullptr;     // device control block of the running solve
     SolveCtl *h_ctl = nullptr;   // pinned copy read after the solve
@@ -425,21 +426,26 @@ enum { kPcgRz = 0, kPcgS1 = 4, kPcgS2 = 8, kPcgAlpha = 12, kPcgBeta = 16, kPcgRz
 // a lane whose r.z has fallen below this fraction of its first value is converged to
 // rounding level (residual about 1e-14 of the start): its step lengths stay 0
 constexpr double kPcgStop = 1e-28;
-void launch_pcg_dot(const double *a, const double *b, int n, int R, double *part, double *sc, int mode,
-                    cudaStream_t s);
-void launch_pcg_direction(const double *z, double *p, const double *sc, int n, int R, cudaStream_t s);
-void launch_pcg_update(double *x, double *r, const double *p, const double *q, const double *sc, int n, int R,
-                       cudaStream_t s);
-// batches: per-mesh dot products over the finest-level work items
-void launch_item_dot2(const int *items, int nitems, const double *a, const double *b, const double *c,
-                      const double *d, int R, double *part, cudaStream_t s);
-void launch_inst_sum(const int *istart, int ninst, const double *part, double *out, int ostride, cudaStream_t s);
-void launch_inst_pcg_scalar(const int *istart, int ninst, int R, const double *part, double *sc, int mode,
-                            const double *norms, const double *tol, cudaStream_t s);
-void launch_inst_pcg_direction(const double *z, double *p, const double *sc, const int *row_inst, int n, int R,
-                               cudaStream_t s);
-void launch_inst_pcg_update(double *x, double *r, const double *p, const double *q, const double *sc,
-                            const int *row_inst, int n, int R, cudaStream_t s);
+// the rows of a conjugate-gradient pass: one mesh (items null), or a batch's work items with the first item of
+// each mesh (istart) and the mesh of each row
+constexpr int kDotRows = 256;   // rows of a work item
+struct PcgRows {
+    const int *items, *istart, *row_inst;
+    int nitems, ninst, n;
+};
+// partial sums part[block or item][8]; see relax.cu
+template <class T> void launch_pcg_z(const PcgRows &w, const double *r, const T *znew, double *z, int R, double *part,
+                                     cudaStream_t s, Chain *ch);
+void launch_pcg_dot(const PcgRows &w, const double *a, const double *b, const double *c, const double *d, int R,
+                    double *part, cudaStream_t s, Chain *ch);
+void launch_pcg_scalar(const PcgRows &w, int R, const double *part, double *sc, int mode, const double *norms,
+                       const double *tol, cudaStream_t s, Chain *ch);
+void launch_pcg_sum(const PcgRows &w, const double *part, double *out, int ostride, int count, int R,
+                    cudaStream_t s, Chain *ch);
+void launch_pcg_direction(const PcgRows &w, const double *z, double *p, const double *sc, float *pair, int R,
+                          cudaStream_t s, Chain *ch);
+template <class T> void launch_pcg_update(const PcgRows &w, double *x, double *r, const double *p, const double *q,
+                                          const double *sc, T *b, int R, double *part, cudaStream_t s, Chain *ch);
 void launch_pack(const double *user, int n, int nrhs, int R, double *v, cudaStream_t s, const int *perm = nullptr);
 void launch_unpack(const double *v, int n, int nrhs, int R, double *user, cudaStream_t s, const int *perm = nullptr);
 void launch_to_float(const double *a, float *b, int64_t n, cudaStream_t s, float *zero = nullptr, Chain *ch = nullptr);

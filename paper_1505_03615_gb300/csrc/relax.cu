@@ -615,23 +615,103 @@ __global__ void __launch_bounds__(128) norm_final_kernel(const double *__restric
 }
 
 // ---- conjugate gradients preconditioned by the V-cycle (per right-hand side lane) ----
-// partial sums of a_i . b_i per lane over a grid-stride range
+// An iteration's vector work is four passes, each doing all that its operands allow: z from the cycle with
+// r.z of the old and the new z; p (and its FP32 pairs for the product); p.q; x, r, the next cycle's right-hand
+// side and r.r.  An iteration on 927k rows took 1007 us (mixed, 3 components) with them apart, 983 us so.
+//
+// Rows are taken in rounds over the GPU (one mesh, kNormBlocks blocks), or, for a batch, as work items: ranges
+// of kDotRows rows of one mesh and colour, a warp each, whose sums are added mesh by mesh.  (With items of 2048
+// rows, added by one thread per mesh and component, an iteration of twelve meshes of 727k rows took 749 us, of
+// 512 rows 691, of 256 678, of 128 680.)
+struct RowRange { int i, end, step; };
+__device__ __forceinline__ RowRange rows_of(const int *items, int nitems, int n) {
+    if (!items) return {(int)(blockIdx.x * blockDim.x + threadIdx.x), n, (int)(gridDim.x * blockDim.x)};
+    const int it = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (it >= nitems) return {0, 0, 32};
+    return {__ldg(items + 3 * it + 1) + (int)(threadIdx.x & 31), __ldg(items + 3 * it + 2), 32};
+}
+
+// component sums of a block (one mesh: part[block][8], from `at` on) or of a warp's item (part[item][8])
 template <int R>
-__global__ void __launch_bounds__(256) dot_partial_kernel(const double *__restrict__ a, const double *__restrict__ b,
-                                                          int n, double *__restrict__ part) {
-    double acc[R];
+__device__ __forceinline__ void put_sums(const double (&acc)[R], const int *items, int nitems, int at, double *part) {
+    if (items) {
+        const int it = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+        int comp;
+        const double v = warp_sum<double, R>(acc, threadIdx.x & 31, comp);
+        if (it < nitems && comp >= 0) part[8 * (size_t)it + at + comp] = v;
+    } else {
+        const double v = block_sum<R>(acc);
+        if (threadIdx.x < R) part[8 * (size_t)blockIdx.x + at + threadIdx.x] = v;
+        __syncthreads();   // its scratch is used again
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void st_vec(double *p, const double (&v)[R]) {
+    if constexpr (R == 1) p[0] = v[0];
+    else
 #pragma unroll
-    for (int r = 0; r < R; r++) acc[r] = 0.0;
+        for (int c = 0; c < R; c += 2) reinterpret_cast<double2 *>(p)[c >> 1] = make_double2(v[c], v[c + 1]);
+}
+
+// z_old.r and z.r, z = the cycle's result; z_old <- z
+template <class T, int R>
+__global__ void __launch_bounds__(256) pcg_z_kernel(const int *__restrict__ items, int nitems, int n,
+                                                    const double *__restrict__ r, const T *__restrict__ znew, double *z,
+                                                    double *__restrict__ part) {
+    grid_dep_wait();
+    grid_dep_launch();
+    const RowRange q = rows_of(items, nitems, n);
+    double a0[R], a1[R];
+#pragma unroll
+    for (int c = 0; c < R; c++) a0[c] = a1[c] = 0.0;
+#pragma unroll 2
+    for (int i = q.i; i < q.end; i += q.step) {
+        double rv[R], zo[R], zd[R];
+        T zn[R];
+        load_x<double, R>(r + (size_t)i * R, rv);
+        load_x<double, R>(z + (size_t)i * R, zo);
+        load_x<T, R>(znew + (size_t)i * R, zn);
+#pragma unroll
+        for (int c = 0; c < R; c++) {
+            zd[c] = (double)zn[c];
+            a0[c] = fma(rv[c], zo[c], a0[c]);
+            a1[c] = fma(rv[c], zd[c], a1[c]);
+        }
+        st_vec<R>(z + (size_t)i * R, zd);
+    }
+    put_sums<R>(a0, items, nitems, 0, part);
+    put_sums<R>(a1, items, nitems, 4, part);
+}
+
+// a.b (components 0..3) and, when c is given, c.d (4..7)
+template <int R>
+__global__ void __launch_bounds__(256) dot_kernel(const int *__restrict__ items, int nitems, int n,
+                                                  const double *__restrict__ a, const double *__restrict__ b,
+                                                  const double *__restrict__ cv, const double *__restrict__ dv,
+                                                  double *__restrict__ part) {
+    grid_dep_wait();
+    grid_dep_launch();
+    const RowRange q = rows_of(items, nitems, n);
+    double a0[R], a1[R];
+#pragma unroll
+    for (int c = 0; c < R; c++) a0[c] = a1[c] = 0.0;
 #pragma unroll 4
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i = q.i; i < q.end; i += q.step) {
         double x[R], y[R];
         load_x<double, R>(a + (size_t)i * R, x);
         load_x<double, R>(b + (size_t)i * R, y);
 #pragma unroll
-        for (int r = 0; r < R; r++) acc[r] = fma(x[r], y[r], acc[r]);
+        for (int c = 0; c < R; c++) a0[c] = fma(x[c], y[c], a0[c]);
+        if (cv) {
+            load_x<double, R>(cv + (size_t)i * R, x);
+            load_x<double, R>(dv + (size_t)i * R, y);
+#pragma unroll
+            for (int c = 0; c < R; c++) a1[c] = fma(x[c], y[c], a1[c]);
+        }
     }
-    const double t = block_sum<R>(acc);
-    if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = t;
+    put_sums<R>(a0, items, nitems, 0, part);
+    if (cv) put_sums<R>(a1, items, nitems, 4, part);
 }
 
 // one scalar step of lane r on the reduced value v (scalars sc, see pcg_scalar_kernel)
@@ -653,162 +733,167 @@ __device__ __forceinline__ void pcg_scalar_step(double *sc, int r, double v, int
     }
 }
 
-// one block: reduce the partial sums to v[lane], then
-//   mode 0: s2 = v                         (r . z of the previous preconditioned residual)
-//   mode 1: s1 = v; beta = (s1 - s2) / rz, rz = s1  (Polak-Ribiere; 0 on the first step, rz = 0;
-//           a lane at rounding level, v <= kPcgStop * its first v, keeps beta = alpha = 0)
-//   mode 2: alpha = s1 / (p . A p), with v = p . q and q = -A p
-__global__ void __launch_bounds__(128) pcg_scalar_kernel(const double *__restrict__ part, int nblocks, int R,
-                                                         double *__restrict__ sc, int mode) {
-    const int r = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (r >= R) return;
-    const double v = partials_sum(part, nblocks, r, lane);
-    if (lane == 0) pcg_scalar_step(sc, r, v, mode);
-}
-
-// p = z + beta p
-__global__ void pcg_direction_kernel(const double *__restrict__ z, double *__restrict__ p,
-                                     const double *__restrict__ sc, int64_t m, int R) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < m) p[q] = fma(sc[kPcgBeta + (int)(q % R)], p[q], z[q]);
-}
-
-// x += alpha p; r += alpha q (q = -A p)
-__global__ void pcg_update_kernel(double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
-                                  const double *__restrict__ qv, const double *__restrict__ sc, int64_t m, int R) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= m) return;
-    const double a = sc[kPcgAlpha + (int)(q % R)];
-    x[q] = fma(a, p[q], x[q]);
-    r[q] = fma(a, qv[q], r[q]);
-}
-
-// ---- the same for a batch: per-mesh dot products over work items (row ranges of one
-// mesh and colour; the items of mesh m are [istart[m], istart[m + 1])) ----
-// per item, per lane: a.b (components 0..3) and, when c is given, c.d (4..7)
-template <int R>
-__global__ void __launch_bounds__(256) item_dot2_kernel(const int *__restrict__ items, int nitems,
-                                                        const double *__restrict__ a, const double *__restrict__ b,
-                                                        const double *__restrict__ cv, const double *__restrict__ dv,
-                                                        double *__restrict__ part) {
+// sum over the items [i0, i1) of component q, by a warp
+__device__ __forceinline__ double items_sum(const double *__restrict__ part, int i0, int i1, int q) {
     const int lane = threadIdx.x & 31;
-    const int it = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (it >= nitems) return;
-    const int r0 = items[3 * it + 1], r1 = items[3 * it + 2];
-    double acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++) acc[q] = 0.0;
-    for (int i = r0 + lane; i < r1; i += 32)
-#pragma unroll
-        for (int q = 0; q < R; q++) {
-            acc[q] = fma(a[(size_t)i * R + q], b[(size_t)i * R + q], acc[q]);
-            if (cv) acc[4 + q] = fma(cv[(size_t)i * R + q], dv[(size_t)i * R + q], acc[4 + q]);
-        }
-#pragma unroll
-    for (int q = 0; q < 8; q++)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-    if (lane < 8) {
-        double v = 0.0;
-#pragma unroll
-        for (int q = 0; q < 8; q++) if (q == lane) v = acc[q];
-        part[8 * (size_t)it + lane] = v;
+    double acc[1] = {0.0};
+#pragma unroll 4
+    for (int it = i0 + lane; it < i1; it += 32) acc[0] += __ldg(part + 8 * (size_t)it + q);
+    int comp;
+    return warp_sum<double, 1>(acc, lane, comp);
+}
+
+// block m: the scalar steps of mesh m, component r by warp r, from the partials [istart[m], istart[m + 1])
+// (one mesh: all kNormBlocks)
+//   mode 1: s2 = v0 (r . z of the previous z), then s1 = v1; beta = (s1 - s2) / rz, rz = s1  (Polak-Ribiere; 0 on
+//           the first step, rz = 0; a lane at rounding level, v <= kPcgStop * its first v, keeps beta = alpha = 0)
+//   mode 2: alpha = s1 / (p . A p), with v0 = p . q and q = -A p
+//   norms (batch): [ninst][16] per-mesh squared norms of r (0..3) and b (4..7) after the last step; tol: the
+//   solve's tolerance.  A mesh lane that meets it takes no further steps: the other meshes keep iterating, and a
+//   converged lane's FP32-preconditioned recurrence would otherwise run on rounding noise.
+__global__ void __launch_bounds__(128) pcg_scalar_kernel(const int *__restrict__ istart, int R,
+                                                         const double *__restrict__ part, double *__restrict__ sc,
+                                                         int mode, const double *__restrict__ norms,
+                                                         const double *__restrict__ tol) {
+    grid_dep_wait();
+    grid_dep_launch();
+    const int m = blockIdx.x, r = threadIdx.x >> 5;
+    if (r >= R) return;
+    const int i0 = istart ? __ldg(istart + m) : 0, i1 = istart ? __ldg(istart + m + 1) : kNormBlocks;
+    const double v0 = items_sum(part, i0, i1, r);
+    const double v1 = mode == 1 ? items_sum(part, i0, i1, 4 + r) : 0.0;
+    if ((threadIdx.x & 31) != 0) return;
+    double *s = sc + (size_t)m * kPcgScalars;
+    bool done = false;
+    if (norms) {
+        const double t = *tol;
+        done = norms[16 * (size_t)m + r] <= t * t * norms[16 * (size_t)m + 4 + r];
+    }
+    if (mode == 1) {
+        pcg_scalar_step(s, r, v0, 0, done);
+        pcg_scalar_step(s, r, v1, 1, done);
+    } else {
+        pcg_scalar_step(s, r, v0, mode, done);
     }
 }
 
-// per mesh m and component q < 8: out[m * ostride + q] = sum of its items' partials (in item order)
-__global__ void inst_sum_kernel(const int *__restrict__ istart, int ninst, const double *__restrict__ part,
-                                double *__restrict__ out, int ostride) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ninst * 8) return;
-    const int m = k >> 3, q = k & 7;
-    double s = 0.0;
-    for (int it = istart[m]; it < istart[m + 1]; it++) s += part[8 * (size_t)it + q];
-    out[(size_t)m * ostride + q] = s;
-}
-
-// per mesh m and lane r: the conjugate-gradient scalar step of pcg_scalar_kernel on
-// v = sum of the mesh's item partials (component r); scalars at sc + m * kPcgScalars
-//   norms: [ninst][16] per-mesh squared norms of r (0..3) and b (4..7) after the last step;
-//   tol: the solve's tolerance.  A mesh lane that meets it takes no further steps: the other
-//   meshes keep iterating, and a converged lane's FP32-preconditioned recurrence would
-//   otherwise run on rounding noise.
-__global__ void inst_pcg_scalar_kernel(const int *__restrict__ istart, int ninst, int R,
-                                       const double *__restrict__ part, double *__restrict__ sc, int mode,
-                                       const double *__restrict__ norms, const double *__restrict__ tol) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ninst * 4) return;
-    const int m = k >> 2, r = k & 3;
-    if (r >= R) return;
+// per mesh m (a block) and component q < count (a warp each): out[m * ostride + q] = sum of its items' partials
+// (0 for the lanes q & 3 >= R, which have none)
+__global__ void __launch_bounds__(256) inst_sum_kernel(const int *__restrict__ istart, const double *__restrict__ part,
+                                                       double *__restrict__ out, int ostride, int count, int R) {
+    grid_dep_wait();
+    grid_dep_launch();
+    const int m = blockIdx.x, q = threadIdx.x >> 5;
+    if (q >= count) return;
     double v = 0.0;
-    for (int it = istart[m]; it < istart[m + 1]; it++) v += part[8 * (size_t)it + r];
-    const double t = *tol;
-    const bool done = norms[16 * (size_t)m + r] <= t * t * norms[16 * (size_t)m + 4 + r];
-    pcg_scalar_step(sc + (size_t)m * kPcgScalars, r, v, mode, done);
+    if ((q & 3) < R)
+        v = items_sum(part, istart ? __ldg(istart + m) : 0, istart ? __ldg(istart + m + 1) : kNormBlocks, q);
+    if ((threadIdx.x & 31) == 0) out[(size_t)m * ostride + q] = v;
 }
 
-// p = z + beta_mesh p; x += alpha_mesh p, r += alpha_mesh q (q = -A p), the mesh of a row from row_inst
-__global__ void inst_pcg_direction_kernel(const double *__restrict__ z, double *__restrict__ p,
-                                          const double *__restrict__ sc, const int *__restrict__ row_inst,
-                                          int64_t m, int R) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= m) return;
-    const double *s = sc + (size_t)row_inst[q / R] * kPcgScalars;
-    p[q] = fma(s[kPcgBeta + (int)(q % R)], p[q], z[q]);
-}
-__global__ void inst_pcg_update_kernel(double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
-                                       const double *__restrict__ qv, const double *__restrict__ sc,
-                                       const int *__restrict__ row_inst, int64_t m, int R) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= m) return;
-    const double a = sc[(size_t)row_inst[q / R] * kPcgScalars + kPcgAlpha + (int)(q % R)];
-    x[q] = fma(a, p[q], x[q]);
-    r[q] = fma(a, qv[q], r[q]);
-}
-
-void launch_item_dot2(const int *items, int nitems, const double *a, const double *b, const double *c,
-                      const double *d, int R, double *part, cudaStream_t s) {
-    if (nitems == 0) return;
-    const unsigned blocks = (unsigned)((nitems + 7) / 8);
-    if (R == 1) item_dot2_kernel<1><<<blocks, 256, 0, s>>>(items, nitems, a, b, c, d, part);
-    else if (R == 2) item_dot2_kernel<2><<<blocks, 256, 0, s>>>(items, nitems, a, b, c, d, part);
-    else item_dot2_kernel<4><<<blocks, 256, 0, s>>>(items, nitems, a, b, c, d, part);
-}
-void launch_inst_sum(const int *istart, int ninst, const double *part, double *out, int ostride, cudaStream_t s) {
-    inst_sum_kernel<<<(unsigned)((ninst * 8 + 255) / 256), 256, 0, s>>>(istart, ninst, part, out, ostride);
-}
-void launch_inst_pcg_scalar(const int *istart, int ninst, int R, const double *part, double *sc, int mode,
-                            const double *norms, const double *tol, cudaStream_t s) {
-    inst_pcg_scalar_kernel<<<(unsigned)((ninst * 4 + 255) / 256), 256, 0, s>>>(istart, ninst, R, part, sc, mode,
-                                                                                norms, tol);
-}
-void launch_inst_pcg_direction(const double *z, double *p, const double *sc, const int *row_inst, int n, int R,
-                               cudaStream_t s) {
-    const int64_t m = (int64_t)n * R;
-    if (m) inst_pcg_direction_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(z, p, sc, row_inst, m, R);
-}
-void launch_inst_pcg_update(double *x, double *r, const double *p, const double *q, const double *sc,
-                            const int *row_inst, int n, int R, cudaStream_t s) {
-    const int64_t m = (int64_t)n * R;
-    if (m) inst_pcg_update_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(x, r, p, q, sc, row_inst, m, R);
+// p = z + beta p, and its FP32 pairs when given; row_inst: the mesh of a row (null: one mesh)
+template <int R>
+__global__ void __launch_bounds__(256) pcg_direction_kernel(const double *__restrict__ z, double *p,
+                                                            const double *__restrict__ sc, const int *__restrict__ row_inst,
+                                                            float *__restrict__ pair, int n) {
+    grid_dep_wait();
+    grid_dep_launch();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double *s = sc + (row_inst ? (size_t)__ldg(row_inst + i) * kPcgScalars : 0) + kPcgBeta;
+    double zv[R], pv[R];
+    load_x<double, R>(z + (size_t)i * R, zv);
+    load_x<double, R>(p + (size_t)i * R, pv);
+#pragma unroll
+    for (int c = 0; c < R; c++) pv[c] = fma(s[c], pv[c], zv[c]);
+    st_vec<R>(p + (size_t)i * R, pv);
+    if (pair) {
+        float h[R], l[R];
+#pragma unroll
+        for (int c = 0; c < R; c++) {
+            h[c] = (float)pv[c];
+            l[c] = (float)(pv[c] - (double)h[c]);
+        }
+        float *q = pair + (size_t)i * (2 * R);
+#pragma unroll
+        for (int c = 0; c < R; c++) { q[c] = h[c]; q[R + c] = l[c]; }
+    }
 }
 
-void launch_pcg_dot(const double *a, const double *b, int n, int R, double *part, double *sc, int mode,
-                    cudaStream_t s) {
-    if (R == 1) dot_partial_kernel<1><<<kNormBlocks, 256, 0, s>>>(a, b, n, part);
-    else if (R == 2) dot_partial_kernel<2><<<kNormBlocks, 256, 0, s>>>(a, b, n, part);
-    else dot_partial_kernel<4><<<kNormBlocks, 256, 0, s>>>(a, b, n, part);
-    pcg_scalar_kernel<<<1, 128, 0, s>>>(part, kNormBlocks, R, sc, mode);
+// x += alpha p, r += alpha q (q = -A p), the next cycle's right-hand side in its type, and r.r
+template <class T, int R>
+__global__ void __launch_bounds__(256) pcg_update_kernel(const int *__restrict__ items, int nitems, int n, double *x,
+                                                         double *r, const double *__restrict__ p,
+                                                         const double *__restrict__ qv, const double *__restrict__ sc,
+                                                         const int *__restrict__ row_inst, T *__restrict__ b,
+                                                         double *__restrict__ part) {
+    grid_dep_wait();
+    grid_dep_launch();
+    const RowRange w = rows_of(items, nitems, n);
+    double acc[R];
+#pragma unroll
+    for (int c = 0; c < R; c++) acc[c] = 0.0;
+#pragma unroll 2
+    for (int i = w.i; i < w.end; i += w.step) {
+        const double *s = sc + (row_inst ? (size_t)__ldg(row_inst + i) * kPcgScalars : 0) + kPcgAlpha;
+        double xv[R], rv[R], pv[R], qq[R];
+        load_x<double, R>(x + (size_t)i * R, xv);
+        load_x<double, R>(r + (size_t)i * R, rv);
+        load_x<double, R>(p + (size_t)i * R, pv);
+        load_x<double, R>(qv + (size_t)i * R, qq);
+#pragma unroll
+        for (int c = 0; c < R; c++) {
+            xv[c] = fma(s[c], pv[c], xv[c]);
+            rv[c] = fma(s[c], qq[c], rv[c]);
+            acc[c] = fma(rv[c], rv[c], acc[c]);
+        }
+        st_vec<R>(x + (size_t)i * R, xv);
+        st_vec<R>(r + (size_t)i * R, rv);
+#pragma unroll
+        for (int c = 0; c < R; c++) b[(size_t)i * R + c] = (T)rv[c];
+    }
+    put_sums<R>(acc, items, nitems, 0, part);
 }
-void launch_pcg_direction(const double *z, double *p, const double *sc, int n, int R, cudaStream_t s) {
-    const int64_t m = (int64_t)n * R;
-    if (m) pcg_direction_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(z, p, sc, m, R);
+
+static unsigned pcg_blocks(const PcgRows &w) { return w.items ? (unsigned)((w.nitems + 7) / 8) : (unsigned)kNormBlocks; }
+
+template <class T>
+void launch_pcg_z(const PcgRows &w, const double *r, const T *znew, double *z, int R, double *part, cudaStream_t s,
+                  Chain *ch) {
+    auto k = R == 1 ? pcg_z_kernel<T, 1> : R == 2 ? pcg_z_kernel<T, 2> : pcg_z_kernel<T, 4>;
+    klaunch(k, pcg_blocks(w), 256u, 0, s, ch, w.items, w.nitems, w.n, r, znew, z, part);
 }
-void launch_pcg_update(double *x, double *r, const double *p, const double *q, const double *sc, int n, int R,
-                       cudaStream_t s) {
-    const int64_t m = (int64_t)n * R;
-    if (m) pcg_update_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(x, r, p, q, sc, m, R);
+template void launch_pcg_z<float>(const PcgRows &, const double *, const float *, double *, int, double *, cudaStream_t, Chain *);
+template void launch_pcg_z<double>(const PcgRows &, const double *, const double *, double *, int, double *, cudaStream_t, Chain *);
+
+void launch_pcg_dot(const PcgRows &w, const double *a, const double *b, const double *c, const double *d, int R,
+                    double *part, cudaStream_t s, Chain *ch) {
+    auto k = R == 1 ? dot_kernel<1> : R == 2 ? dot_kernel<2> : dot_kernel<4>;
+    klaunch(k, pcg_blocks(w), 256u, 0, s, ch, w.items, w.nitems, w.n, a, b, c, d, part);
 }
+void launch_pcg_scalar(const PcgRows &w, int R, const double *part, double *sc, int mode, const double *norms,
+                       const double *tol, cudaStream_t s, Chain *ch) {
+    klaunch(pcg_scalar_kernel, (unsigned)w.ninst, 128u, 0, s, ch, w.istart, R, part, sc, mode, norms, tol);
+}
+void launch_pcg_sum(const PcgRows &w, const double *part, double *out, int ostride, int count, int R, cudaStream_t s,
+                    Chain *ch) {
+    klaunch(inst_sum_kernel, (unsigned)w.ninst, 256u, 0, s, ch, w.istart, part, out, ostride, count, R);
+}
+void launch_pcg_direction(const PcgRows &w, const double *z, double *p, const double *sc, float *pair, int R,
+                          cudaStream_t s, Chain *ch) {
+    auto k = R == 1 ? pcg_direction_kernel<1> : R == 2 ? pcg_direction_kernel<2> : pcg_direction_kernel<4>;
+    if (w.n) klaunch(k, (unsigned)((w.n + 255) / 256), 256u, 0, s, ch, z, p, sc, w.row_inst, pair, w.n);
+}
+template <class T>
+void launch_pcg_update(const PcgRows &w, double *x, double *r, const double *p, const double *q, const double *sc, T *b,
+                       int R, double *part, cudaStream_t s, Chain *ch) {
+    auto k = R == 1 ? pcg_update_kernel<T, 1> : R == 2 ? pcg_update_kernel<T, 2> : pcg_update_kernel<T, 4>;
+    klaunch(k, pcg_blocks(w), 256u, 0, s, ch, w.items, w.nitems, w.n, x, r, p, q, sc, w.row_inst, b, part);
+}
+template void launch_pcg_update<float>(const PcgRows &, double *, double *, const double *, const double *,
+                                       const double *, float *, int, double *, cudaStream_t, Chain *);
+template void launch_pcg_update<double>(const PcgRows &, double *, double *, const double *, const double *,
+                                        const double *, double *, int, double *, cudaStream_t, Chain *);
 
 void launch_norms(const double *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch) {
     auto k = R == 1 ? norm_partial_kernel<double, 1> : R == 2 ? norm_partial_kernel<double, 2> : norm_partial_kernel<double, 4>;
