@@ -67,7 +67,9 @@ typedef struct lbmg_options {
                            bounded waits; always used for batches); 0 (default): one graph launch
                            per cycle */
     int narrow_max;     /* bottom levels with at most this many rows run inside one block, with
-                           block barriers between their phases (default 2048) */
+                           block barriers between their phases (default 2048); where a single mesh's
+                           do not fit in shared memory, or in a batch, only if a level of them is
+                           too small for a tiled sweep */
     int barrier_phantoms; /* fault injection for tests, default 0: the persistent solve's grid barrier
                            waits for this many extra arrivals that never come, so its bounded wait
                            (about one second) expires and lbmg_solve returns LBMG_DEVICE_TIMEOUT */

@@ -300,6 +300,18 @@ bool top_from_zero(const Ctx &c, int d, int R) {
             (c.smoother == LBMG_GS_COLOURED && !tiled<T>(c, L, R) && sweeps_from_zero<T>(L)));
 }
 
+// Whether the levels above d0, up to d, go in one block that reads global memory.  Not where all of them are
+// tiled: twelve meshes' levels of 271 and 1358 rows took 130 us in one block and 30 us as seven launches (a
+// CG iteration of the batch 683 us and 587 us).  Single meshes' bottoms start from shared memory instead.
+template <class T>
+bool one_block(const Ctx &c, int d, int R) {
+    if (d < c.d0) return false;
+    if (!(c.nu1 > 0 && c.nu2 > 0)) return true;
+    for (int l = c.d0 + 1; l <= d; l++)
+        if (!tiled<T>(c, c.lev[l], R)) return true;
+    return false;
+}
+
 // Tiled levels take a launch or two per sweep, the residual with the last sweep down, the prolongation in
 // the first one up (timed: the events bracket these too).
 // zero: e is zero on entry (the tiled finest level does not read it then).
@@ -313,7 +325,7 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
     enum { kPlain, kSmem, kL2 } bottom = kPlain;
     if (sizeof(T) == 4 && c.smoother != LBMG_JACOBI) {
         if (c.narrow.dn >= c.d0 && c.narrow.dn <= top) { bottom = kSmem; dn = c.narrow.dn; }
-        else if (std::min(c.persist_dn, top) >= c.d0) { bottom = kL2; dn = std::min(c.persist_dn, top); }
+        else if (one_block<T>(c, std::min(c.persist_dn, top), R)) { bottom = kL2; dn = std::min(c.persist_dn, top); }
     }
     int skip = 0;   // colour steps of the next level's first sweep that its restriction did
     TileVec<T> vec[kMaxDepth + 1];
@@ -1916,7 +1928,7 @@ int lbmg_launch_counts(lbmg_handle h, int precision, int *assemble, int *project
     };
     int cyc = 0;
     if (c.gamma == 1 && !c.coarse_smooth) {
-        const bool narrow = c.persist_dn >= c.d0 && c.smoother != LBMG_JACOBI && precision == LBMG_MIXED;
+        const bool narrow = one_block<float>(c, c.persist_dn, 4) && c.smoother != LBMG_JACOBI && precision == LBMG_MIXED;
         const bool smem = c.narrow.dn >= c.d0 && c.smoother != LBMG_JACOBI && precision == LBMG_MIXED;
         const int bottom = smem ? c.narrow.dn : (narrow ? c.persist_dn : c.d0);
         cyc = 1;   // the one-block bottom cycle, or the coarse apply
