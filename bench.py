@@ -828,6 +828,8 @@ def main():
         tpr, tpb = shapes[str(D)][0]
         kname = "pk_row_kernel" if tpr == 4 else "smooth_colour_kernel"
         kernel = f"{kname}<float,{R},GS> (finest level, one colour, {tpr} threads per row, {tpb} threads/block)"
+        if (tpr, tpb) == (4, 256) and n <= 80_000:   # the default shape stands for the tiled sweep there
+            kernel = f"tile_kernel<float,{R}> (finest level; an eighth of a sweep, transfers of its launches included)"
         key = f"{kname}_gs_{workload}"
     achieved = launch_bytes / (avg_launch_ms * 1e-3) / 1e9 if avg_launch_ms > 0 else 0.0
     traffic = None

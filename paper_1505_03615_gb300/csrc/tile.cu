@@ -17,7 +17,8 @@
 // sweep of torus-knot levels, colour launches / tiles: 18 / 5.5 us at 5,000 rows, 18 / 7.5 at 19,000, 18 / 11
 // at 78,000, 28 / 27 at 232,000, 76 / 71-79 at 927,000; a cycle of the 1M-triangle sheets with four
 // components took 1410 us with 91,000 rows tiled, 1283 without.  FP64 at three right-hand sides: 42 / 14 us,
-// 42 / 30, 42 / 37, 60 / 70, 290 / 310.
+// 42 / 30, 42 / 37, 60 / 70, 290 / 310, with colour launches that summed the padding lane too; without it the
+// line still holds (a cycle of the 200k knot 608 us with it at 60,000 rows, 632 with it at 15,000).
 //
 // Four lanes share a row, as in packed.cu, so that a row's gathers are few per lane and all in flight
 // together (a step is one chain of shared-memory latencies); the lanes' sums are added so that lane c ends
