@@ -287,19 +287,6 @@ inline void record(cudaEvent_t e, cudaStream_t s, Chain *ch) {
     ch->cut();
 }
 
-// one V-cycle on A e = b at the finest level; e (finest x) must be zero on entry.
-// Every coarser correction is zeroed by the restriction that fills its right-hand
-// side, so the kernels of the cycle follow one another with no memset between
-// them and run as one chain of dependent launches.
-// whether a V-cycle from zero on level d reads nothing of its x before it has written it
-template <class T>
-bool top_from_zero(const Ctx &c, int d, int R) {
-    const DevLevel &L = c.lev[d];
-    return c.gamma == 1 && !c.coarse_smooth && c.nu1 > 0 && d > c.d0 &&
-           ((tiled<T>(c, L, R) && c.nu2 > 0) ||
-            (c.smoother == LBMG_GS_COLOURED && !tiled<T>(c, L, R) && sweeps_from_zero<T>(L)));
-}
-
 // Whether the levels above d0, up to d, go in one block that reads global memory.  Not where all of them are
 // tiled: twelve meshes' levels of 271 and 1358 rows took 130 us in one block and 30 us as seven launches (a
 // CG iteration of the batch 683 us and 587 us).  Single meshes' bottoms start from shared memory instead.
@@ -312,21 +299,44 @@ bool one_block(const Ctx &c, int d, int R) {
     return false;
 }
 
+// The bottom levels of a cycle with finest level `top`: from shared memory in one block (FP32), from global
+// memory in one block (levels of at most narrow_max rows), or one launch per phase down to d0 (a single SM's
+// FP64 rate makes the one-block bottom slower than per-phase launches).  dn: the highest of them.
+enum class Bottom { kPlain, kSmem, kL2 };
+template <class T>
+Bottom bottom_of(const Ctx &c, int top, int R, int *dn) {
+    *dn = c.d0;
+    if (sizeof(T) == 4 && c.smoother != LBMG_JACOBI) {
+        if (c.narrow.dn >= c.d0 && c.narrow.dn <= top) { *dn = c.narrow.dn; return Bottom::kSmem; }
+        const int low = std::min(c.persist_dn, top);
+        if (one_block<T>(c, low, R)) { *dn = low; return Bottom::kL2; }
+    }
+    return Bottom::kPlain;
+}
+
+// Whether a V-cycle from zero on level d reads nothing of its x before it has written it.  (The one block that
+// reads global memory sweeps its top level as it finds it; the one in shared memory starts from zero itself.)
+template <class T>
+bool top_from_zero(const Ctx &c, int d, int R) {
+    const DevLevel &L = c.lev[d];
+    int dn;
+    if (bottom_of<T>(c, d, R, &dn) == Bottom::kL2 && dn == d) return false;
+    return c.gamma == 1 && !c.coarse_smooth && c.nu1 > 0 && d > c.d0 &&
+           ((tiled<T>(c, L, R) && c.nu2 > 0) ||
+            (c.smoother == LBMG_GS_COLOURED && !tiled<T>(c, L, R) && sweeps_from_zero<T>(L)));
+}
+
+// One V-cycle on A e = b at the finest level (or at `top`).  Every coarser correction is zeroed by the
+// restriction that fills its right-hand side, so the kernels of the cycle follow one another with no memset
+// between them and run as one chain of dependent launches.
 // Tiled levels take a launch or two per sweep, the residual with the last sweep down, the prolongation in
 // the first one up (timed: the events bracket these too).
-// zero: e is zero on entry (the tiled finest level does not read it then).
+// zero_start: e counts as zero; it has to be zero on entry unless top_from_zero() says that it is not read.
 template <class T>
 void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int top = -1, bool zero_start = true) {
     if (top < 0) top = c.D;
-    // bottom levels: from shared memory in one block (FP32), from global memory in
-    // one block (levels of at most narrow_max rows), or one launch per phase down to d0
-    // (a single SM's FP64 rate makes the one-block bottom slower than per-phase launches)
-    int dn = c.d0;
-    enum { kPlain, kSmem, kL2 } bottom = kPlain;
-    if (sizeof(T) == 4 && c.smoother != LBMG_JACOBI) {
-        if (c.narrow.dn >= c.d0 && c.narrow.dn <= top) { bottom = kSmem; dn = c.narrow.dn; }
-        else if (one_block<T>(c, std::min(c.persist_dn, top), R)) { bottom = kL2; dn = std::min(c.persist_dn, top); }
-    }
+    int dn;
+    const Bottom bottom = bottom_of<T>(c, top, R, &dn);
     int skip = 0;   // colour steps of the next level's first sweep that its restriction did
     TileVec<T> vec[kMaxDepth + 1];
     auto tile = [&](int d) { return c.nu1 > 0 && c.nu2 > 0 && tiled<T>(c, c.lev[d], R); };
@@ -355,15 +365,16 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
         }
         // the shared-memory bottom starts level dn from zero itself; the dense solve overwrites d0
         // (and a tiled level's first sweep starts from zero without reading it)
-        const bool zero = (bottom == kSmem ? d - 1 > dn : (bottom == kL2 || d - 1 > c.d0)) && !(d - 1 > dn && tile(d - 1));
+        const bool zero = (bottom == Bottom::kSmem ? d - 1 > dn : (bottom == Bottom::kL2 || d - 1 > c.d0)) &&
+                          !(d - 1 > dn && tile(d - 1));
         // a level that this loop smooths next (Gauss-Seidel, from zero) gets its first colour step
         // from the restriction that zeroes it
         const bool fuse = zero && d - 1 > dn && c.smoother != LBMG_JACOBI && c.nu1 > 0;
         launch_restrict<T>(Lc, P<T>::r(L), P<T>::b(Lc), R, s, zero ? P<T>::x(Lc) : (T *)nullptr, ch, fuse);
         skip = fuse ? 1 : 0;
     }
-    if (bottom == kSmem) launch_narrow_smem(c, R, s, ch);
-    else if (bottom == kL2) { launch_narrow_cycle(c, 1, R, dn, s); ch->cut(); }
+    if (bottom == Bottom::kSmem) launch_narrow_smem(c, R, s, ch);
+    else if (bottom == Bottom::kL2) { launch_narrow_cycle(c, 1, R, dn, s); ch->cut(); }
     else {
         DevLevel &L0 = c.lev[c.d0];
         launch_coarse_apply<T>(c, L0, P<T>::inv(c), P<T>::b(L0), P<T>::x(L0), R, s, ch);
