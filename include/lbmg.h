@@ -48,8 +48,8 @@ enum {
     LBMG_COARSE_FACTOR = 6,    /* coarsest-level Cholesky met a non-positive pivot */
     LBMG_CUDA_ERROR = 7,       /* a CUDA call failed; lbmg_last_cuda_error() names it */
     LBMG_DIVERGED = 8,         /* residual became NaN or grew by 1e6 */
-    LBMG_DEVICE_TIMEOUT = 9    /* a bounded device-side wait (grid barrier, or the bottom kernel's copy of
-                                  its static data) expired; results are invalid */
+    LBMG_DEVICE_TIMEOUT = 9    /* a bounded device-side wait (grid barrier, step barrier of a tiled sweep,
+                                  or a kernel's copy of its static data) expired; results are invalid */
 };
 
 enum { LBMG_FP64 = 0, LBMG_MIXED = 1 };          /* precision of the V-cycle */
@@ -71,8 +71,9 @@ typedef struct lbmg_options {
                            do not fit in shared memory, or in a batch, only if a level of them is
                            too small for a tiled sweep */
     int barrier_phantoms; /* fault injection for tests, default 0: the persistent solve's grid barrier
-                           waits for this many extra arrivals that never come, so its bounded wait
-                           (about one second) expires and lbmg_solve returns LBMG_DEVICE_TIMEOUT */
+                           and the step barriers of tiled sweeps wait for this many extra arrivals that
+                           never come, so their bounded waits (about one second; 10 ms in tiled sweeps)
+                           expire and lbmg_solve returns LBMG_DEVICE_TIMEOUT */
     int use_graphs;     /* per-cycle path: 1 (default) replays a captured CUDA graph per cycle; 0
                            launches the cycle's kernels directly (same kernels, e.g. for profilers) */
     int pdl;            /* per-cycle path: 1 (default) chains the cycle's kernels with programmatic

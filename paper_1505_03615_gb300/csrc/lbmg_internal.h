@@ -259,7 +259,7 @@ struct Ctx {
     int pdl = 1;                  // chain the kernels of a cycle with programmatic dependent launch
     int persist_ok = 0;
     int persist_blocks = 0, persist_dn = 0, persist_narrow = 2048;
-    int barrier_phantoms = 0;        // fault injection: extra arrivals a grid barrier waits for
+    int barrier_phantoms = 0;        // fault injection: extra arrivals a grid barrier or a tiled sweep's step waits for
     int copy_phantoms = 0;           // fault injection: extra bytes the bottom kernel's copy waits for
     void *persist_views = nullptr;
     void *views32 = nullptr, *views64 = nullptr;   // level views for the one-block bottom cycle

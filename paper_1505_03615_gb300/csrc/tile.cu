@@ -37,7 +37,8 @@ namespace {
 
 constexpr int kTileWarps = 8, kTileThreads = 32 * kTileWarps;
 constexpr int kTileRing = 16;                                 // groups in flight per warp at most
-constexpr unsigned long long kTileWaitNs = 1000000000ull;     // a copy is given up after one second
+// a copy or a step's barrier is given up after one second; after 10 ms where arrivals are missing on purpose
+constexpr unsigned long long kTileWaitNs = 1000000000ull, kTilePhantomWaitNs = 10000000ull;
 
 template <int N> struct Int { static constexpr int value = N; };
 template <class T> struct TileCfg;
@@ -65,7 +66,9 @@ struct TileArgs {
     const int *par;
     const int8_t *npl2;
     T *r;
-    int *status;               // set to 1 when a copy did not arrive in time
+    int *status;               // set to 1 when a copy or a warp did not arrive in time
+    int arrivals;              // of a step's barrier: the warps, and in a test more that never come
+    unsigned long long wait_ns;
 };
 
 // a row of R components, in one or two vector accesses
@@ -124,8 +127,9 @@ __device__ __forceinline__ unsigned long long tile_now() {
     return t;
 }
 
-// waits for the barrier's phase, at most kTileWaitNs
-__device__ __forceinline__ bool tile_wait(uint32_t mbar, uint32_t parity) {
+// waits for the barrier's phase, at most wait_ns by the lane's own clock: lanes may disagree, so what a warp
+// does next has to follow from all of them
+__device__ __forceinline__ bool tile_wait(uint32_t mbar, uint32_t parity, unsigned long long wait_ns) {
     unsigned long long t0 = 0;
     for (;;) {
         uint32_t done;
@@ -137,7 +141,7 @@ __device__ __forceinline__ bool tile_wait(uint32_t mbar, uint32_t parity) {
         if (done) return true;
         const unsigned long long t = tile_now();
         if (t0 == 0) t0 = t;
-        else if (t - t0 > kTileWaitNs) return false;
+        else if (t - t0 > wait_ns) return false;
     }
 }
 
@@ -156,7 +160,7 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? 3 : 2) tile_ker
     if (tid < kTileInfo) s_info[tid] = __ldg(a.info + (size_t)blockIdx.x * kTileInfo + tid);
     if (tid == 0)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_step)),
-                     "r"(kTileWarps)
+                     "r"(a.arrivals)
                      : "memory");
     if (tid < kTileWarps * a.ring) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(s_bar + tid))
@@ -242,14 +246,14 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? 3 : 2) tile_ker
     T d = T(0), bv = T(0), v[KP];
     bool ok = true, stale = false;
     auto place = [&]() { return ring + (size_t)(warp * a.ring + at) * a.gbytes; };
-    auto arrived = [&]() { return tile_wait((uint32_t)__cvta_generic_to_shared(s_bar + warp * a.ring + at), phase); };
+    auto arrived = [&]() { return tile_wait((uint32_t)__cvta_generic_to_shared(s_bar + warp * a.ring + at), phase, a.wait_ns); };
     auto read_ahead = [&]() {
         stale = false;
         if (g >= gend || !ok) return;
         K = scum[g + 1] - scum[g];
         if (!__all_sync(kFull, arrived())) {
             ok = false;
-            atomicExch(a.status, 1);
+            if (lane == 0) atomicExch(a.status, 1);
             return;
         }
         const unsigned char *p = place(), *e = p + kHead<T>;
@@ -349,7 +353,12 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? 3 : 2) tile_ker
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sbar) : "memory");
         e = s_info[5 + s + 1];
         if (stale) { read_ahead(); rhs(); }
-        if (!tile_wait(sbar, s & 1)) { ok = false; atomicExch(a.status, 1); }
+        // (the whole warp gives up, or none of it: the loops above take the lanes together; it still arrives at
+        // the steps that are left, but waits for nobody any more)
+        if (ok && !__all_sync(kFull, tile_wait(sbar, s & 1, a.wait_ns))) {
+            ok = false;
+            if (lane == 0) atomicExch(a.status, 1);
+        }
     }
     if (a.nsteps > 0)
         for (int i = tid; i < nown; i += kTileThreads) {
@@ -526,7 +535,7 @@ void launch_tile_fill(const DevLevel &L, cudaStream_t s) {
 
 template <class T>
 static void launch_tile(const DevLevel &L, const TileDev &t, int part, const TileVec<T> &v, const T *b, T *r, int R,
-                        int lanes, int *status, cudaStream_t s, Chain *ch) {
+                        const Ctx &c, cudaStream_t s, Chain *ch) {
     TileArgs<T> a;
     a.info = t.info; a.loc = t.loc; a.cum = t.cum; a.stream = tile_stream<T>(t);
     a.nsteps = t.nsteps; a.maxloc = t.maxloc; a.maxcomp = t.maxcomp; a.maxgrp = t.maxgrp;
@@ -540,9 +549,11 @@ static void launch_tile(const DevLevel &L, const TileDev &t, int part, const Til
     for (int q = 0; q + 1 < kTileParts; q++) a.bound[q] = q + 1 < L.tparts ? L.cs[(q + 1) * per] : L.n;
     a.xout = ((v.cur >> part) & 1u) ? v.x : v.y;
     a.xc = v.xc; a.par = L.par; a.npl2 = L.npl2; a.r = r;
-    a.status = status;
+    a.status = c.narrow.status;
+    a.arrivals = kTileWarps + c.barrier_phantoms;
+    a.wait_ns = c.barrier_phantoms > 0 ? kTilePhantomWaitNs : kTileWaitNs;
     auto k = R == 1 ? tile_kernel<T, 1, 1> : R == 2 ? tile_kernel<T, 2, 2>
-             : lanes == 3 ? tile_kernel<T, 4, 3> : tile_kernel<T, 4, 4>;
+             : c.lanes == 3 ? tile_kernel<T, 4, 3> : tile_kernel<T, 4, 4>;
     klaunch(k, (unsigned)t.ntile, (unsigned)kTileThreads, tile_smem<T>(t, R, a.ring), s, ch, a);
 }
 
@@ -552,12 +563,12 @@ void launch_tile_sweep(const Ctx &c, const DevLevel &L, bool forward, TileVec<T>
     const int dir = forward ? 0 : 1;
     for (int q = 0; q < L.tparts; q++) {
         const int part = forward ? q : L.tparts - 1 - q;
-        launch_tile<T>(L, L.tile[dir][part], part, v, b, L.tfused ? r : (T *)nullptr, R, c.lanes, c.narrow.status, s, ch);
+        launch_tile<T>(L, L.tile[dir][part], part, v, b, L.tfused ? r : (T *)nullptr, R, c, s, ch);
         v.cur ^= 1u << part;
         v.zero &= ~(1u << part);
         v.prolong &= ~(1u << part);
     }
-    if (r && !L.tfused) launch_tile<T>(L, L.tres, 0, v, b, r, R, c.lanes, c.narrow.status, s, ch);
+    if (r && !L.tfused) launch_tile<T>(L, L.tres, 0, v, b, r, R, c, s, ch);
 }
 
 template void launch_tile_sweep<float>(const Ctx &, const DevLevel &, bool, TileVec<float> &, const float *, float *, int,
