@@ -49,7 +49,11 @@ enum {
     LBMG_CUDA_ERROR = 7,       /* a CUDA call failed; lbmg_last_cuda_error() names it */
     LBMG_DIVERGED = 8,         /* residual became NaN or grew by 1e6 */
     LBMG_DEVICE_TIMEOUT = 9    /* a bounded device-side wait (grid barrier, step barrier of a tiled sweep,
-                                  or a kernel's copy of its static data) expired; results are invalid */
+                                  or a kernel's copy of its static data) expired; results are invalid.
+                                  A call that does not wait for the device (lbmg_smooth, and lbmg_vcycles
+                                  with use_graphs = 0 or host_check = 1, on device pointers) returns before
+                                  the wait can expire: the next solve, smoothing on host arrays, eigenpair,
+                                  tuning or training call on the handle reports it then, once */
 };
 
 enum { LBMG_FP64 = 0, LBMG_MIXED = 1 };          /* precision of the V-cycle */
@@ -309,7 +313,7 @@ int lbmg_cmcf_step(lbmg_handle h, const double *X, double delta, double *x, doub
  *  *iters: iterations taken.  The call allocates and frees its work blocks (about
  *  9 k n doubles).  Errors: LBMG_NOT_ASSEMBLED, LBMG_INVALID_ARG (sizes, host pointers, a
  *  batch), LBMG_DIVERGED (the block lost rank), LBMG_NOT_CONVERGED (x, lambda hold the last
- *  iterate), LBMG_CUDA_ERROR.
+ *  iterate), LBMG_DEVICE_TIMEOUT, LBMG_CUDA_ERROR.
  */
 int lbmg_eigs(lbmg_handle h, int k, double tol, int max_iters, const double *X0, double *lambda, double *X,
               double *residuals, int *iters, void *stream);
@@ -514,6 +518,8 @@ int lbmg_host_row_instances(lbmg_host_handle h, int d, int *inst);
  *    receives each step's mean loss.
  *  lbmg_learned_enable: on = 1 puts the correction in front of every cycle of this
  *    handle's solves (its stencil features follow each lbmg_assemble); 0 removes it.
+ *  The three training calls return LBMG_DEVICE_TIMEOUT when a bounded wait of their
+ *    cycles expired (lbmg_learned_collect then stores no samples).
  *  lbmg_learned_apply: the correction of one residual r [n_depth][ns] (ns <= 4) by
  *    the solve's own kernels in the given precision (LBMG_MIXED: FP32 features and
  *    start, LBMG_FP64: FP64): omega [n_depth] and delta [n_depth][ns], user order.

@@ -665,19 +665,12 @@ int get_cond_graph(lbmg_handle h, int R, int precision, bool pcg, cudaGraphExec_
 }
 
 int read_norms(lbmg_handle h, int R, cudaStream_t s, double *out4) {
-    // four norms, then the bottom kernel's status word
+    // four norms, then the word of the bounded waits
     LBMG_CK(cudaMemcpyAsync(h->c.h_norm, h->c.norm_out, 5 * sizeof(double), cudaMemcpyDeviceToHost, s));
     LBMG_CK(cudaStreamSynchronize(s));
     h->syncs++;
     for (int r = 0; r < 4; r++) out4[r] = r < R ? h->c.h_norm[r] : 0.0;
-    int st = 0;
-    std::memcpy(&st, &h->c.h_norm[4], sizeof st);
-    if (st != 0) {
-        // a bounded wait in the bottom kernel gave up: the cycle's result is invalid
-        LBMG_CK(cudaMemsetAsync(h->c.norm_out + 4, 0, sizeof(double), s));
-        return LBMG_DEVICE_TIMEOUT;
-    }
-    return LBMG_OK;
+    return timeout_taken(h->c, s) ? LBMG_DEVICE_TIMEOUT : LBMG_OK;
 }
 
 int check_level(lbmg_handle h, int d) {
@@ -1002,6 +995,16 @@ int upload_hierarchy(lbmg_handle h) {
 }  // namespace
 
 namespace lbmg {
+cudaError_t timeout_fetch(const Ctx &c, cudaStream_t s) {
+    return cudaMemcpyAsync(c.h_norm + 4, c.norm_out + 4, sizeof(double), cudaMemcpyDeviceToHost, s);
+}
+bool timeout_taken(const Ctx &c, cudaStream_t s) {
+    int st = 0;
+    std::memcpy(&st, &c.h_norm[4], sizeof st);
+    if (st != 0) cudaMemsetAsync(c.norm_out + 4, 0, sizeof(double), s);
+    return st != 0;
+}
+
 void enqueue_vcycle64_from(Ctx &c, int top, int R, cudaStream_t s) {
     Chain ch;   // plain launches
     enqueue_vcycle<double>(c, R, s, false, &ch, top);
@@ -1494,10 +1497,12 @@ static int solve_pcg_batch(lbmg_handle h, const double *rd, const double *xin, d
     nh.assign(16 * (size_t)c.ninst, 0.0);
     h->syncs = 0;
     auto read = [&]() -> int {
+        LBMG_CK(timeout_fetch(c, s));
         LBMG_CK(cudaMemcpyAsync(nh.data(), c.inst_norm, nh.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
         LBMG_CK(cudaStreamSynchronize(s));
         h->syncs++;
-        return check_launch();
+        LBMG_TRY(check_launch());
+        return timeout_taken(c, s) ? LBMG_DEVICE_TIMEOUT : LBMG_OK;
     };
     auto worst = [&](const std::vector<double> &v, double *w) {
         for (int r = 0; r < 4; r++) w[r] = 0.0;
@@ -1586,6 +1591,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
         LBMG_CK(cudaMemcpyAsync(hs, c.persist_state, 64, cudaMemcpyDeviceToHost, s));
         LBMG_CK(cudaMemcpyAsync(h->h_inst, c.inst_norm, 16 * sizeof(double) * c.ninst, cudaMemcpyDeviceToHost, s));
         LBMG_CK(cudaMemcpyAsync(h->h_flag, c.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+        LBMG_CK(timeout_fetch(c, s));   // of an earlier call that did not wait
         launch_unpack(c.xs, Fl.n, nrhs, R, xout, s, c.fperm);
         LBMG_CK(cudaEventRecord(c.ev1, s));
         h->syncs = 0;
@@ -1611,7 +1617,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
                 worst0[r] = std::max(worst0[r], rel0);
             }
         int status = LBMG_OK;
-        if (dstat == 1) status = LBMG_DEVICE_TIMEOUT;
+        if (timeout_taken(c, s) || dstat == 1) status = LBMG_DEVICE_TIMEOUT;
         else if (*h->h_flag != 0) status = LBMG_COARSE_FACTOR;
         else if (dstat == 2) status = LBMG_DIVERGED;
         else if (check && !conv) status = LBMG_NOT_CONVERGED;
@@ -1730,9 +1736,12 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
     if (pairs) launch_join(c.xs_pair, c.xs, Fl.n, R, s);
     launch_unpack(c.xs, Fl.n, nrhs, R, xout, s, c.fperm);
     LBMG_CK(cudaEventRecord(c.ev1, s));
+    // (a stopping test has read the word with the last norms)
+    const bool waits = !check && (host_out || stats);
+    if (waits) LBMG_CK(timeout_fetch(c, s));
     LBMG_TRY(finish_output(x, xout, cnt, host_out, s, &h->syncs));
     if (stats) {
-        LBMG_CK(cudaEventSynchronize(c.ev1));
+        LBMG_CK(waits ? cudaStreamSynchronize(s) : cudaEventSynchronize(c.ev1));
         if (!host_out) h->syncs++;
         float ms = 0;
         cudaEventElapsedTime(&ms, c.ev0, c.ev1);
@@ -1743,7 +1752,7 @@ static int solve_impl(lbmg_handle h, const double *rhs, double *x, int nrhs, dou
         stats->learned_fallback = dropped ? 1 : 0;
         if (!check) stats->cycles = cycles;
     }
-    return status;
+    return waits && timeout_taken(c, s) ? LBMG_DEVICE_TIMEOUT : status;
 }
 
 int lbmg_cmcf_step(lbmg_handle h, const double *X, double delta, double *x, double tol, int max_cycles,
@@ -1788,6 +1797,7 @@ int lbmg_eigs(lbmg_handle h, int k, double tol, int max_iters, const double *X0,
         case 0: return LBMG_OK;
         case 1: return LBMG_INVALID_ARG;
         case 2: return LBMG_CUDA_ERROR;
+        case 5: return LBMG_DEVICE_TIMEOUT;
         case 3: return LBMG_DIVERGED;
         default: return LBMG_NOT_CONVERGED;
     }
@@ -1885,7 +1895,10 @@ int lbmg_smooth(lbmg_handle h, int d, const double *rhs, double *x, int nrhs, in
     bool host_out;
     LBMG_TRY(output_ptr(h, x, cnt, 1, &xo, &host_out));
     launch_unpack(L.x64, L.n, nrhs, R, xo, s);
-    return finish_output(x, xo, cnt, host_out, s);
+    if (host_out) LBMG_CK(timeout_fetch(h->c, s));
+    LBMG_TRY(finish_output(x, xo, cnt, host_out, s));
+    // (device pointers: nothing waits here, the next call that does reports)
+    return host_out && timeout_taken(h->c, s) ? LBMG_DEVICE_TIMEOUT : LBMG_OK;
 }
 
 int lbmg_restrict(lbmg_handle h, int d, const double *r_fine, double *r_coarse, int nrhs, void *stream) {
@@ -1986,7 +1999,9 @@ int lbmg_autotune(lbmg_handle h, int nrhs, int precision, int reps, int *timed, 
         cudaGetLastError();
         return LBMG_CUDA_ERROR;
     }
-    return LBMG_OK;
+    LBMG_CK(timeout_fetch(c, (cudaStream_t)stream));
+    LBMG_CK(cudaStreamSynchronize((cudaStream_t)stream));
+    return timeout_taken(c, (cudaStream_t)stream) ? LBMG_DEVICE_TIMEOUT : LBMG_OK;
 }
 
 int lbmg_launch_shape(lbmg_handle h, int d, int precision, int *out) {
@@ -2057,6 +2072,16 @@ static int learned_ready(lbmg_handle h, cudaStream_t s) {
     return LBMG_OK;
 }
 
+// what learned.cu's training calls return (0, 1: argument, 2: CUDA, 3: a bounded wait gave up)
+static int learned_status(int st) {
+    switch (st) {
+        case 0: return LBMG_OK;
+        case 1: return LBMG_INVALID_ARG;
+        case 3: return LBMG_DEVICE_TIMEOUT;
+        default: return LBMG_CUDA_ERROR;
+    }
+}
+
 int lbmg_learned_nparams(void) { return learned_nparams(); }
 
 int lbmg_learned_params(lbmg_handle h, double *get, const double *set, void *stream) {
@@ -2080,7 +2105,7 @@ int lbmg_learned_collect(lbmg_handle h, const double *rhs, int ns, int skip, int
     const size_t cnt = (size_t)h->c.lev[h->c.D].n * ns;
     if (!on_device(rhs) && cnt > h->io_cap) return LBMG_INVALID_ARG;
     LBMG_TRY(input_ptr(h, rhs, cnt, 0, s, &rd));
-    return learned_collect(h->c, rd, ns, skip, keep, s) ? LBMG_CUDA_ERROR : LBMG_OK;
+    return learned_status(learned_collect(h->c, rd, ns, skip, keep, s));
 }
 
 int lbmg_learned_loss_grad(lbmg_handle h, const double *r0, int ns, double *loss, double *grad, void *stream) {
@@ -2089,7 +2114,7 @@ int lbmg_learned_loss_grad(lbmg_handle h, const double *r0, int ns, double *loss
     LBMG_TRY(learned_ready(h, s));
     const double *rd;
     LBMG_TRY(input_ptr(h, r0, (size_t)h->c.lev[h->c.D].n * ns, 0, s, &rd));
-    return learned_loss_grad(h->c, rd, ns, loss, grad, s) ? LBMG_CUDA_ERROR : LBMG_OK;
+    return learned_status(learned_loss_grad(h->c, rd, ns, loss, grad, s));
 }
 
 int lbmg_learned_train(lbmg_handle h, int steps, double lr, const int *order, int batch, double *loss_hist,
@@ -2097,8 +2122,7 @@ int lbmg_learned_train(lbmg_handle h, int steps, double lr, const int *order, in
     cudaStream_t s = (cudaStream_t)stream;
     if (steps < 0 || !order || batch < 1 || batch > 8 || !(lr > 0)) return LBMG_INVALID_ARG;
     LBMG_TRY(learned_ready(h, s));
-    const int st = learned_train(h->c, steps, lr, order, batch, loss_hist, s);
-    return st == 1 ? LBMG_INVALID_ARG : (st ? LBMG_CUDA_ERROR : LBMG_OK);
+    return learned_status(learned_train(h->c, steps, lr, order, batch, loss_hist, s));
 }
 
 int lbmg_learned_enable(lbmg_handle h, int on, void *stream) {

@@ -319,9 +319,14 @@ size_t persist_view_bytes();
 void launch_cmcf_weights(const Ctx &c, const double *X, double *tri_w, cudaStream_t s);
 
 // ----- smallest eigenpairs of L x = lambda M x (lobpcg.cu) -----
-// 0 converged, 1 bad size, 2 CUDA failure, 3 the block lost rank, 4 not converged in max_iters
+// 0 converged, 1 bad size, 2 CUDA failure, 3 the block lost rank, 4 not converged in max_iters, 5 a bounded wait gave up
 int lobpcg(Ctx &c, int k, double tol, int max_iters, const double *X_user, double *lambda, double *X_out, double *res,
            int *iters, cudaStream_t s, std::string &err);
+
+// The word that a kernel sets when one of its bounded waits gives up (NarrowState::status), for calls that wait
+// for the device anyway: fetched with their other results, before the wait; taken (and cleared) after it.
+cudaError_t timeout_fetch(const Ctx &c, cudaStream_t s);
+bool timeout_taken(const Ctx &c, cudaStream_t s);
 
 // ----- kernels (assemble.cu) -----
 void launch_fragment_moments(const Ctx &c, cudaStream_t s);

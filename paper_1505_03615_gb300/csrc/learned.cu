@@ -696,6 +696,13 @@ static void sample_pass(Ctx &c, bool need_grad, double weight, bool accumulate, 
     grad_reduce_kernel<<<(kNP + 255) / 256, 256, 0, s>>>(L->part_blocks, L->part, accumulate ? 1 : 0, L->grad);
 }
 
+// end of a training call: 0, 2 (CUDA) or 3 (a bounded wait of its cycles gave up, its results are invalid)
+static int finish_training(Ctx &c, cudaStream_t s) {
+    if (timeout_fetch(c, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess)
+        return 2;
+    return timeout_taken(c, s) ? 3 : 0;
+}
+
 static int ensure_loss(Learned *L, int count) {
     if (count <= L->loss_cap) return 0;
     if (L->loss_dev) cudaFree(L->loss_dev);
@@ -715,7 +722,7 @@ int learned_loss_grad(Ctx &c, const double *r0_user, int ns, double *loss, doubl
     if (cudaMemcpyAsync(loss, L->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess) return 2;
     if (grad && cudaMemcpyAsync(grad, L->grad, sizeof(double) * kNP, cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return 2;
-    return cudaStreamSynchronize(s) == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : 2;
+    return finish_training(c, s);
 }
 
 // residual histories of plain FP64 V-cycles from x = 0 on the columns of rhs ([n][ns] user
@@ -752,8 +759,9 @@ int learned_collect(Ctx &c, const double *rhs_user, int ns, int skip, int keep, 
         enqueue_vcycle64_from(c, c.D, 4, s);
         launch_add_double(x, F.x64, m4, s);
     }
-    L->bank_n += keep;
-    return cudaStreamSynchronize(s) == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : 2;
+    const int st = finish_training(c, s);
+    if (st == 0) L->bank_n += keep;
+    return st;
 }
 
 // Adam steps over bank samples; order: host [steps][batch] sample indices; the step's
@@ -780,7 +788,7 @@ int learned_train(Ctx &c, int steps, double lr, const int *order, int batch, dou
     if (steps > 0 &&
         cudaMemcpyAsync(lh.data(), L->loss_dev, sizeof(double) * steps * batch, cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return 2;
-    if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return 2;
+    if (const int st = finish_training(c, s)) return st;
     if (loss_hist)
         for (int it = 0; it < steps; it++) {
             double a = 0.0;

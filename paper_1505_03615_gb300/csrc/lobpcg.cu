@@ -299,9 +299,13 @@ int lobpcg(Ctx &c, int k, double tol, int max_iters, const double *X_user, doubl
         gram(m, w.U, m, w.MU, w.G + (size_t)m * m);
         if ((e = cudaMemcpyAsync(host.data(), w.G, host.size() * sizeof(double), cudaMemcpyDeviceToHost, s)) !=
                 cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess) {
+            (e = timeout_fetch(c, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess) {
             err = std::string("lbmg_eigs: ") + cudaGetErrorString(e);
             return 2;
+        }
+        if (timeout_taken(c, s)) {   // of the V-cycles that gave this basis
+            err = "lbmg_eigs: a bounded device wait gave up";
+            return 5;
         }
         GL.assign(host.begin(), host.begin() + (size_t)m * m);
         GM.assign(host.begin() + (size_t)m * m, host.end());
