@@ -1046,6 +1046,19 @@ static int check_build_options(const lbmg_options &o) {
     return LBMG_OK;
 }
 
+// the upload, whose plans and tables take host memory: nothing is thrown through a C entry
+static int upload_guarded(lbmg_handle h) {
+    try {
+        return upload_hierarchy(h);
+    } catch (const std::bad_alloc &) {
+        g_cuda_err = "hierarchy upload: host memory exhausted";
+        return LBMG_OUT_OF_MEMORY;
+    } catch (const std::exception &e) {
+        g_cuda_err = std::string("hierarchy upload: ") + e.what();
+        return LBMG_INVALID_ARG;
+    }
+}
+
 // host hierarchy of one mesh in the layout the device handle uploads; on failure the
 // reason goes to the thread's error string
 static int build_single_host(const double *V, int nv, const int *F, int nt, int depth, const lbmg_options &o,
@@ -1235,7 +1248,7 @@ int lbmg_build_hierarchy(const double *V, int nv, const int *F, int nt, int dept
     h->c.host_check = o.host_check;
     h->c.gamma = o.cycle == 1 ? 2 : 1;
     h->c.coarse_smooth = o.coarse_smooth;
-    st = upload_hierarchy(h);
+    st = upload_guarded(h);
     if (st != 0) { delete h; return st; }
     *out = h;
     return LBMG_OK;
@@ -1259,7 +1272,7 @@ int lbmg_build_batch(const double *const *V, const int *nv, const int *const *F,
     h->c.nu1 = o.nu1; h->c.nu2 = o.nu2; h->c.smoother = o.smoother; h->c.omega = o.jacobi_omega;
     h->c.persistent = 1; h->c.persist_narrow = o.narrow_max; h->c.barrier_phantoms = o.barrier_phantoms;
     h->c.host_check = o.host_check;
-    st = upload_hierarchy(h);
+    st = upload_guarded(h);
     if (st != 0) { delete h; return st; }
     if (!h->c.persist_ok) { delete h; return LBMG_CUDA_ERROR; }
     *out = h;

@@ -9,7 +9,9 @@
 // read from the level's vector.  With colours by corner parity a sweep reaches at most 7, 3 and 1
 // corners along the axes, so on surfaces the overlap is a thin rim of the tile.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
+#include <new>
 #include <numeric>
 
 #include "tile_plan.h"
@@ -20,19 +22,38 @@ namespace {
 
 using Block = TileCut::Block;
 
+// A host allocation that fails inside a parallel region or a task: remembered there (an exception that leaves
+// one ends the process) and thrown by the caller's thread behind it.
+struct AllocFailure {
+    std::atomic<bool> failed{false};
+    template <class F>
+    void guard(F &&work) {
+        if (failed) return;
+        try {
+            work();
+        } catch (...) {
+            failed = true;
+        }
+    }
+    void rethrow() const {
+        if (failed) throw std::bad_alloc();
+    }
+};
+
 // The steps reach over at most 7 (x), 3 (y) and 1 (z) corners, the residual and the rim's own reads over
 // one or two more: tiles are cut across the axis along which they measure the most reaches.
 constexpr int kReach[3] = {8, 4, 2};
 
 // blocks [b0, b1) into ntile tiles from t0 on, by recursive bisection at equal shares of entries
-void bisect(std::vector<Block> &blk, int64_t b0, int64_t b1, int t0, int ntile, std::vector<int64_t> &start) {
+void bisect(std::vector<Block> &blk, int64_t b0, int64_t b1, int t0, int ntile, std::vector<int64_t> &start,
+            AllocFailure &alloc) {
     if (ntile <= 1) {
         start[t0] = b0;
         return;
     }
     const int tl = ntile / 2;
     int64_t m = b0;
-    if (b1 > b0) {
+    auto cut = [&]() {
         int lo[3], hi[3], il = blk[b0].inst, ih = il;
         for (int a = 0; a < 3; a++) lo[a] = hi[a] = blk[b0].at[a];
         double w = 0;
@@ -60,20 +81,23 @@ void bisect(std::vector<Block> &blk, int64_t b0, int64_t b1, int t0, int ntile, 
         const int ay = ax == 0 ? ((int64_t)(hi[1] - lo[1] + 1) * kReach[2] >= (int64_t)(hi[2] - lo[2] + 1) * kReach[1] ? 1 : 2) : 0;
         std::stable_sort(mid, end, [&](const Block &A, const Block &B) { return A.at[ay] < B.at[ay]; });
         for (; m < end - blk.begin() && acc + blk[m].weight <= left; m++) acc += blk[m].weight;
-    }
+    };
+    if (b1 > b0) alloc.guard(cut);
     const int64_t mm = m;
-#pragma omp task shared(blk, start) if (b1 - b0 > 4096)
-    bisect(blk, b0, mm, t0, tl, start);
-#pragma omp task shared(blk, start) if (b1 - b0 > 4096)
-    bisect(blk, mm, b1, t0 + tl, ntile - tl, start);
+#pragma omp task shared(blk, start, alloc) if (b1 - b0 > 4096)
+    bisect(blk, b0, mm, t0, tl, start, alloc);
+#pragma omp task shared(blk, start, alloc) if (b1 - b0 > 4096)
+    bisect(blk, mm, b1, t0 + tl, ntile - tl, start, alloc);
 #pragma omp taskwait
 }
 
 void bisect_all(TileCut &cut, int ntile) {
     cut.start.assign(ntile + 1, (int64_t)cut.blocks.size());
+    AllocFailure alloc;
 #pragma omp parallel
 #pragma omp single
-    bisect(cut.blocks, 0, (int64_t)cut.blocks.size(), 0, ntile, cut.start);
+    bisect(cut.blocks, 0, (int64_t)cut.blocks.size(), 0, ntile, cut.start, alloc);
+    alloc.rethrow();
 }
 
 struct TileOut {
@@ -141,7 +165,9 @@ bool split_tiles(const TilePlan &plan, int maxloc, TileCut &cut) {
     for (int t = 0; t < plan.ntile; t++) {
         start.push_back(cut.start[t]);
         if (plan.info[(size_t)t * kTileInfo] <= maxloc || cut.start[t + 1] - cut.start[t] < 2) continue;
-        bisect(cut.blocks, cut.start[t], cut.start[t + 1], 0, 2, half);
+        AllocFailure alloc;
+        bisect(cut.blocks, cut.start[t], cut.start[t + 1], 0, 2, half, alloc);
+        alloc.rethrow();
         if (half[1] > cut.start[t] && half[1] < cut.start[t + 1]) { start.push_back(half[1]); any = true; }
     }
     start.push_back(cut.start[plan.ntile]);
@@ -160,12 +186,15 @@ bool build_tile_plan(const HostLevel &L, const TileCut &cut, const int *seq, int
     for (int s = 0; s < nsteps; s++) steps_colour[seq[s]] = true;
     std::vector<uint8_t> colour(L.ns);
     for (int c = 0; c < 8; c++) std::fill(colour.begin() + L.colour_start[c], colour.begin() + L.colour_start[c + 1], (uint8_t)c);
+    AllocFailure alloc;
 #pragma omp parallel
     {
-        std::vector<int32_t> mark(L.ndof, -1), slot_of(L.ndof, 0);
-        std::vector<int32_t> list[8], order;
-#pragma omp for schedule(dynamic, 1)
-        for (int t = 0; t < ntile; t++) {
+        std::vector<int32_t> mark, slot_of, list[8], order;
+        alloc.guard([&]() {
+            mark.assign(L.ndof, -1);
+            slot_of.assign(L.ndof, 0);
+        });
+        auto one = [&](int t) {
             TileOut &T = tiles[t];
             size_t own[8], cnt[kTileSteps], comp[8] = {0};   // needed rows at each step, computed rows of each colour
             for (int c = 0; c < 8; c++) {
@@ -214,7 +243,7 @@ bool build_tile_plan(const HostLevel &L, const TileCut &cut, const int *seq, int
                 std::sort(order.begin(), order.end());
                 T.loc.insert(T.loc.end(), order.begin(), order.end());
             }
-            if (T.loc.size() > 65534) { T.ok = false; continue; }
+            if (T.loc.size() > 65534) { T.ok = false; return; }
             for (size_t q = 0; q < T.loc.size(); q++) slot_of[T.loc[q]] = (int32_t)q;
             // groups of kTileRows rows, longest rows first, so that a group's rows are about equally long
             auto len = [&](int i) { return L.rp[i + 1] - L.rp[i]; };
@@ -255,8 +284,11 @@ bool build_tile_plan(const HostLevel &L, const TileCut &cut, const int *seq, int
                 groups(order);
             }
             T.step_end[nsteps] = (int32_t)T.gk.size();
-        }
+        };
+#pragma omp for schedule(dynamic, 1)
+        for (int t = 0; t < ntile; t++) alloc.guard([&]() { one(t); });
     }
+    alloc.rethrow();
     for (const TileOut &T : tiles)
         if (!T.ok) return false;
     std::vector<int64_t> g0(ntile + 1, 0), q0(ntile + 1, 0);
