@@ -38,7 +38,7 @@ namespace {
 constexpr int kTileWarps = 8, kTileThreads = 32 * kTileWarps;
 constexpr int kTileRing = 16;                                 // groups in flight per warp at most
 // a copy or a step's barrier is given up after one second; after 10 ms where arrivals are missing on purpose
-constexpr unsigned long long kTileWaitNs = 1000000000ull, kTilePhantomWaitNs = 10000000ull;
+constexpr unsigned kTileWaitNs = 1000000000u, kTilePhantomWaitNs = 10000000u;
 
 template <int N> struct Int { static constexpr int value = N; };
 template <class T> struct TileCfg;
@@ -68,7 +68,7 @@ struct TileArgs {
     T *r;
     int *status;               // set to 1 when a copy or a warp did not arrive in time
     int arrivals;              // of a step's barrier: the warps, and in a test more that never come
-    unsigned long long wait_ns;
+    unsigned wait_ns;          // bound of every wait
 };
 
 // a row of R components, in one or two vector accesses
@@ -121,16 +121,17 @@ __device__ __forceinline__ void copy_row_async(T *dst, const T *src) {
     }
 }
 
-__device__ __forceinline__ unsigned long long tile_now() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+__device__ __forceinline__ unsigned tile_now() {   // (differences of up to four seconds)
+    unsigned t;
+    asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
     return t;
 }
 
-// waits for the barrier's phase, at most wait_ns by the lane's own clock: lanes may disagree, so what a warp
-// does next has to follow from all of them
-__device__ __forceinline__ bool tile_wait(uint32_t mbar, uint32_t parity, unsigned long long wait_ns) {
-    unsigned long long t0 = 0;
+// waits for the barrier's phase, at most wait_ns by the lane's own clock: lanes may disagree, so no control
+// flow that the lanes of a warp take together may follow from one lane's answer
+__device__ __forceinline__ bool tile_wait(uint32_t mbar, uint32_t parity, unsigned wait_ns) {
+    unsigned t0 = 0;
+    bool first = true;
     for (;;) {
         uint32_t done;
         asm volatile(
@@ -139,9 +140,9 @@ __device__ __forceinline__ bool tile_wait(uint32_t mbar, uint32_t parity, unsign
             : "r"(mbar), "r"(parity)
             : "memory");
         if (done) return true;
-        const unsigned long long t = tile_now();
-        if (t0 == 0) t0 = t;
-        else if (t - t0 > wait_ns) return false;
+        const unsigned t = tile_now();
+        if (first) { t0 = t; first = false; }
+        if (t - t0 >= wait_ns) return false;
     }
 }
 
@@ -336,6 +337,7 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? 3 : 2) tile_ker
         if (g < e) { read_ahead(); rhs(); }
     };
     const uint32_t sbar = (uint32_t)__cvta_generic_to_shared(&s_step);
+    unsigned step_ns = a.wait_ns;
     read_ahead();
     copies_done();
     __syncthreads();
@@ -353,11 +355,11 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? 3 : 2) tile_ker
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sbar) : "memory");
         e = s_info[5 + s + 1];
         if (stale) { read_ahead(); rhs(); }
-        // (the whole warp gives up, or none of it: the loops above take the lanes together; it still arrives at
-        // the steps that are left, but waits for nobody any more)
-        if (ok && !__all_sync(kFull, tile_wait(sbar, s & 1, a.wait_ns))) {
-            ok = false;
-            if (lane == 0) atomicExch(a.status, 1);
+        // A lane whose wait expires goes on with the others (the loops above take the lanes of a warp together):
+        // what it reads is invalid but in place, and it does not wait at the steps that are left.
+        if (!tile_wait(sbar, s & 1, step_ns)) {
+            step_ns = 0;
+            atomicExch(a.status, 1);
         }
     }
     if (a.nsteps > 0)
