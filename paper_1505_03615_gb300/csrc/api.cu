@@ -487,9 +487,10 @@ void enqueue_iteration(Ctx &c, int R, int precision, cudaStream_t s, bool timed 
                 launch_packed_residual_split(F, c.bs, c.xs_pair, c.rs, R, s, &ch);
                 launch_norms(c.rs, F.n, R, c.norm_part, c.norm_out, s, &ch);
             } else {
-                launch_packed_outer(F, c.bs3, c.xs_pair, F.b32, top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32, R,
-                                    c.lanes, s, &ch);
-                launch_norms32(F.b32, F.n, R, c.norm_part, c.norm_out, s, &ch);
+                // (the low parts, for the norms only, in the residual's place of the cycle)
+                launch_packed_outer(F, c.bs3, c.xs_pair, F.b32, F.r32,
+                                    top_from_zero<float>(c, c.D, R) ? (float *)nullptr : F.x32, R, c.lanes, s, &ch);
+                launch_norms_pair(F.b32, F.r32, F.n, R, c.norm_part, c.norm_out, s, &ch);
             }
             return;
         }

@@ -359,10 +359,10 @@ template <class T> bool launch_packed_residual(const DevLevel &L, const T *A, co
 // bits) and b - sum in FP64; false when the level has no packed copy
 bool launch_packed_residual_split(const DevLevel &L, const double *b, const float *xp, double *r, int R,
                                   cudaStream_t s, Chain *ch);
-// the same at the end of a mixed iteration: b as three FP32 numbers (launch_split3), the result in FP32
-// (r32; z zeroed when given)
-bool launch_packed_outer(const DevLevel &L, const float4 *b3, const float *xp, float *r32, float *z, int R, int lanes,
-                         cudaStream_t s, Chain *ch);
+// the same at the end of a mixed iteration: b as three FP32 numbers (launch_split3), the result as an FP32 pair
+// (r32 + rlo; z zeroed when given)
+bool launch_packed_outer(const DevLevel &L, const float4 *b3, const float *xp, float *r32, float *rlo, float *z, int R,
+                         int lanes, cudaStream_t s, Chain *ch);
 void launch_split3(const double *x, float4 *out, int64_t n, cudaStream_t s);
 // the pairs of an FP64 vector (xp may be x); x = hi + lo in FP64; x += e on the pairs (FP32 two-sum)
 void launch_split(const double *x, float *xp, int n, int R, cudaStream_t s);
@@ -425,7 +425,8 @@ template <class T> void launch_coarse_apply(const Ctx &c, const DevLevel &L, con
 void launch_coarse_factor(const Ctx &c, const int *const *rps, const int *const *cis, const double *const *As,
                           cudaStream_t s);
 void launch_norms(const double *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch = nullptr);
-void launch_norms32(const float *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch = nullptr);
+void launch_norms_pair(const float *hi, const float *lo, int n, int R, double *part, double *out, cudaStream_t s,
+                       Chain *ch = nullptr);
 // conjugate-gradient scalars in Ctx::pcg_s, four lanes each
 enum { kPcgRz = 0, kPcgS1 = 4, kPcgS2 = 8, kPcgAlpha = 12, kPcgBeta = 16, kPcgRz0 = 20, kPcgScalars = 24 };
 // a lane whose r.z has fallen below this fraction of its first value is converged to

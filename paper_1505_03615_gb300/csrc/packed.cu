@@ -319,16 +319,19 @@ __global__ void __launch_bounds__(256) pk_split_residual_kernel(int g1, const in
     }
 }
 
-// The same residual at the end of a mixed V-cycle iteration: r rounded to FP32, the next cycle's right-hand
-// side (z, when given, zeroed as its start).  The right-hand side comes as three FP32 numbers (53 bits) and is
+// The same residual at the end of a mixed V-cycle iteration, as an FP32 pair: r rounded to FP32, the next cycle's
+// right-hand side (z, when given, zeroed as its start), and what the rounding left (rlo), which the norms need:
+// of r rounded alone they were off by up to 1e-8 of themselves on some hundred rows.  The right-hand side comes
+// as three FP32 numbers (53 bits, down to FP32's smallest numbers, where the products' pairs end too) and is
 // subtracted as pairs, so that no FP64 instruction is left (a warp issues one in about 64 cycles).  The norms
-// are a pass of their own over r32: summed here, the FP64 additions at every block's end held its place
+// are a pass of their own over r32 and rlo: summed here, the FP64 additions at every block's end held its place
 // (94 -> 140 us).  NC of the R components are live.
 template <int R, int NC>
 __global__ void __launch_bounds__(256) pk_outer_kernel(int g1, const int2 *__restrict__ gq, const int *__restrict__ rows,
                                                        const int *__restrict__ col, const float2 *__restrict__ v2,
                                                        const float4 *__restrict__ b3, const float *__restrict__ xp,
-                                                       float *__restrict__ r32, float *__restrict__ z) {
+                                                       float *__restrict__ r32, float *__restrict__ rlo,
+                                                       float *__restrict__ z) {
     const int lane = threadIdx.x & 31, l = lane & 3;
     const int g = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
     if (g >= g1) return;   // whole warps only
@@ -399,14 +402,18 @@ __global__ void __launch_bounds__(256) pk_outer_kernel(int g1, const int2 *__res
     }
     if (row >= 0 && l < R) {
         const size_t q = (size_t)row * R + l;
-        float rr = 0.f;
+        float rr = 0.f, rl = 0.f;
         if (l < NC) {
             const float4 b = __ldg(b3 + q);
-            float s2, e2;
+            float s2, e2, p, pe, q2, qe;
             two_sum(b.x, -h, s2, e2);
-            rr = __fadd_rn(s2, __fadd_rn(__fadd_rn(e2, __fsub_rn(b.y, lo)), b.z));
+            two_sum(b.y, -lo, p, pe);
+            two_sum(e2, p, q2, qe);
+            two_sum(s2, q2, rr, rl);
+            rl = __fadd_rn(rl, __fadd_rn(__fadd_rn(qe, pe), b.z));
         }
         r32[q] = rr;
+        rlo[q] = rl;
         if (z) z[q] = 0.f;
     }
 }
@@ -757,14 +764,14 @@ void launch_join(const float *xp, double *x, int n, int R, cudaStream_t s) {
     if (m) join_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(xp, x, m, R);
 }
 
-bool launch_packed_outer(const DevLevel &L, const float4 *b3, const float *xp, float *r32, float *z, int R, int lanes,
-                         cudaStream_t s, Chain *ch) {
+bool launch_packed_outer(const DevLevel &L, const float4 *b3, const float *xp, float *r32, float *rlo, float *z, int R,
+                         int lanes, cudaStream_t s, Chain *ch) {
     if (!L.pk_map || !L.pk_v2) return false;
     auto k = R == 1 ? pk_outer_kernel<1, 1> : R == 2 ? pk_outer_kernel<2, 2>
              : lanes == 3 ? pk_outer_kernel<4, 3> : pk_outer_kernel<4, 4>;
     if (L.pk_gs[9] <= 0) return true;
     klaunch(k, (unsigned)(((int64_t)L.pk_gs[9] * 32 + 255) / 256), 256u, 0, s, ch, L.pk_gs[9], (const int2 *)L.pk_gq, (const int *)L.pk_rows,
-            (const int *)L.pk_col, (const float2 *)L.pk_v2, b3, xp, r32, z);
+            (const int *)L.pk_col, (const float2 *)L.pk_v2, b3, xp, r32, rlo, z);
     return true;
 }
 

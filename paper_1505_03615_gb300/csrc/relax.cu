@@ -562,13 +562,15 @@ void launch_coarse_factor(const Ctx &c, const int *const *rps, const int *const 
 }
 
 // ---- per-right-hand-side sums of squares, two passes (deterministic) ----
-// the block's sum of each component: per warp, then over the warps; thread c < R returns component c
+// the block's sum of each component: per warp, then over the warps; thread c < R returns component c.
+// rest, when given: FP32 sums of each component to be added with the weight w
 template <int R>
-__device__ __forceinline__ double block_sum(const double (&acc)[R]) {
+__device__ __forceinline__ double block_sum(const double (&acc)[R], const float (*rest)[R] = nullptr, double w = 0.0) {
     __shared__ double sh[8][4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int comp;
-    const double v = warp_sum<double, R>(acc, lane, comp);
+    double v = warp_sum<double, R>(acc, lane, comp);
+    if (rest) v = fma((double)warp_sum<float, R>(*rest, lane, comp), w, v);
     if (comp >= 0) sh[warp][comp] = v;
     __syncthreads();
     double t = 0.0;
@@ -579,8 +581,8 @@ __device__ __forceinline__ double block_sum(const double (&acc)[R]) {
 
 // One round of blocks over the GPU, a row's components in one or two vector loads.  (256 blocks and scalar
 // loads took 38 us for 927k rows of four components, 30 MB.)
-template <class T, int R>
-__global__ void __launch_bounds__(256) norm_partial_kernel(const T *__restrict__ v, int n, double *__restrict__ part) {
+template <int R>
+__global__ void __launch_bounds__(256) norm_partial_kernel(const double *__restrict__ v, int n, double *__restrict__ part) {
     grid_dep_wait();
     grid_dep_launch();
     double acc[R];
@@ -588,12 +590,84 @@ __global__ void __launch_bounds__(256) norm_partial_kernel(const T *__restrict__
     for (int r = 0; r < R; r++) acc[r] = 0.0;
 #pragma unroll 4
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        T x[R];
-        load_x<T, R>(v + (size_t)i * R, x);
+        double x[R];
+        load_x<double, R>(v + (size_t)i * R, x);
 #pragma unroll
-        for (int r = 0; r < R; r++) acc[r] = fma((double)x[r], (double)x[r], acc[r]);
+        for (int r = 0; r < R; r++) acc[r] = fma(x[r], x[r], acc[r]);
     }
     const double t = block_sum<R>(acc);
+    if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = t;
+}
+
+// The same for a vector of FP32 pairs: (hi + lo)^2 = hi^2 + (2 hi + lo) lo, hi^2 in FP64 and the rest, at most 2^-23
+// of it, in FP32 sums, scaled by 2^64 against underflow.  The FP64 pipe's instructions are the time (6 us each for
+// 927k rows of four components; all in FP64, four of them, it took 32.5 us), so hi is widened by moving its bits.
+// Numbers for which the FP32 range might not hold (below 2^-85 or from 2^30 on, but for zero) take the FP64 way.
+constexpr float kPairScale = 1.8446744073709552e19f;   // 2^64
+
+__device__ __forceinline__ double pair_sum(float hi, float lo) {   // (volatile: not before its branch is taken)
+    double h, l;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(h) : "f"(hi));
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(l) : "f"(lo));
+    return h + l;
+}
+
+template <int R>
+__global__ void __launch_bounds__(256) norm_pair_partial_kernel(const float *__restrict__ hi, const float *__restrict__ lo,
+                                                                int n, double *__restrict__ part) {
+    grid_dep_wait();
+    grid_dep_launch();
+    if ((int)(blockIdx.x * blockDim.x) >= n) {   // no rows (the sums alone take some FP64 time)
+        if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = 0.0;
+        return;
+    }
+    constexpr int U = R == 4 ? 2 : 4;   // rows in flight
+    double acc[R];
+    float rest[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) { acc[r] = 0.0; rest[r] = 0.f; }
+    const int step = gridDim.x * blockDim.x;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += U * step) {
+        float h[U][R], l[U][R];
+        bool usual = true;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (u == 0 || i + u * (int64_t)step < n) {
+                load_x<float, R>(hi + (size_t)(i + u * (int64_t)step) * R, h[u]);
+                load_x<float, R>(lo + (size_t)(i + u * (int64_t)step) * R, l[u]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; r++) h[u][r] = l[u][r] = 0.f;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+#pragma unroll
+            for (int r = 0; r < R; r++) {
+                const unsigned a = __float_as_uint(h[u][r]) & 0x7fffffffu;   // |hi|
+                usual = usual && (a - 0x15000000u < 0x39800000u || (a == 0u && l[u][r] == 0.f));
+            }
+        if (usual) {
+#pragma unroll
+            for (int u = 0; u < U; u++)
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const unsigned a = __float_as_uint(h[u][r]) & 0x7fffffffu;
+                    const double d = __hiloint2double(a ? (int)((a >> 3) + 0x38000000u) : 0, (int)(a << 29));
+                    acc[r] = fma(d, d, acc[r]);
+                    rest[r] = fmaf(fmaf(2.f, h[u][r], l[u][r]), l[u][r] * kPairScale, rest[r]);
+                }
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; u++)
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const double d = pair_sum(h[u][r], l[u][r]);
+                    acc[r] = fma(d, d, acc[r]);
+                }
+        }
+    }
+    const double t = block_sum<R>(acc, &rest, 1.0 / (double)kPairScale);
     if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = t;
 }
 
@@ -896,13 +970,14 @@ template void launch_pcg_update<double>(const PcgRows &, double *, double *, con
                                         const double *, double *, int, double *, cudaStream_t, Chain *);
 
 void launch_norms(const double *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch) {
-    auto k = R == 1 ? norm_partial_kernel<double, 1> : R == 2 ? norm_partial_kernel<double, 2> : norm_partial_kernel<double, 4>;
+    auto k = R == 1 ? norm_partial_kernel<1> : R == 2 ? norm_partial_kernel<2> : norm_partial_kernel<4>;
     klaunch(k, (unsigned)kNormBlocks, 256u, 0, s, ch, v, n, part);
     klaunch(norm_final_kernel, 1u, 128u, 0, s, ch, (const double *)part, (int)kNormBlocks, R, out);
 }
-void launch_norms32(const float *v, int n, int R, double *part, double *out, cudaStream_t s, Chain *ch) {
-    auto k = R == 1 ? norm_partial_kernel<float, 1> : R == 2 ? norm_partial_kernel<float, 2> : norm_partial_kernel<float, 4>;
-    klaunch(k, (unsigned)kNormBlocks, 256u, 0, s, ch, v, n, part);
+void launch_norms_pair(const float *hi, const float *lo, int n, int R, double *part, double *out, cudaStream_t s,
+                       Chain *ch) {
+    auto k = R == 1 ? norm_pair_partial_kernel<1> : R == 2 ? norm_pair_partial_kernel<2> : norm_pair_partial_kernel<4>;
+    klaunch(k, (unsigned)kNormBlocks, 256u, 0, s, ch, hi, lo, n, part);
     klaunch(norm_final_kernel, 1u, 128u, 0, s, ch, (const double *)part, (int)kNormBlocks, R, out);
 }
 
