@@ -368,7 +368,9 @@ int lbmg_set_launch_shape(lbmg_handle h, int d, int precision, int kind, int tpr
 int lbmg_set_host_check(lbmg_handle h, int on);
 /* write / read the process-wide tuning cache as text, one entry per line:
    device fp64 kind lanes rows nnz threads_per_row threads_per_block [grid], the last the
-   whole-sweep kernel's blocks, or -1 for the tiled sweep.
+   whole-sweep kernel's blocks, or -1 for the tiled sweep.  Lines without it, and files whose
+   header ends with [sweep_grid] (saved before there were tiled sweeps), leave open whether a
+   level's sweeps are tiled.
    Load merges valid lines and returns LBMG_INVALID_ARG if the file cannot be
    opened or a line is malformed (valid lines are still taken). */
 int lbmg_tune_cache_save(const char *path);

@@ -21,6 +21,7 @@ struct LaunchShape {
     int tpr = 4, tpb = 256;   // Gauss-Seidel with tpb = 1024: the whole-sweep cooperative kernel (packed.cu)
     int grid = 0;             // its blocks (0: one per SM; fewer make the grid barrier cheaper on small levels)
     bool tile = true;         // the tiled kernel (tile.cu) where the level has a plan; tpr, tpb are then unused
+    bool keep_tile = false;   // (a tuning entry that knew no tiles: the level's `tile` stays as it is)
 };
 constexpr int kSweepShapeTpb = 1024;
 enum { kShapeSmooth = 0, kShapeResidual = 1 };

@@ -10,6 +10,7 @@
 // (device name, precision, kernel, lanes, rows, non-zeros), which can be saved to
 // and loaded from a text file.
 #include <cstdio>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <string>
@@ -114,7 +115,9 @@ cudaError_t tune_levels(Ctx &c, int R, int reps, int *timed) {
                 std::lock_guard<std::mutex> lk(g_mu);
                 auto it = g_cache.find(key);
                 if (it != g_cache.end()) {
+                    const bool tile = L.shape[fp64][kind].tile;
                     L.shape[fp64][kind] = it->second;
+                    if (it->second.keep_tile) L.shape[fp64][kind].tile = tile;
                     L.tuned_ms[fp64][kind] = 0.f;
                     continue;
                 }
@@ -203,16 +206,27 @@ int autotune(Ctx &c, int R, int precision, int reps, cudaStream_t s, int *timed)
     return (int)e;
 }
 
+// Files saved when there were colour shapes only: their shapes won against no tiles, so they leave open whether
+// a level's sweeps are tiled (as the oldest files' lines do, which end with the threads per block).
+static const char *const kHeadNoTiles = "[sweep_grid]";
+
 int tune_cache_save(const char *path) {
     FILE *f = std::fopen(path, "w");
     if (!f) return 1;
     std::lock_guard<std::mutex> lk(g_mu);
-    std::fprintf(f, "# device fp64 kind lanes rows nnz threads_per_row threads_per_block [sweep_grid, -1: tiled sweep]\n");
-    for (const auto &kv : g_cache) {
-        const Key &k = kv.first;
-        std::fprintf(f, "%s %d %d %d %lld %lld %d %d %d\n", std::get<0>(k).c_str(), std::get<1>(k), std::get<2>(k),
-                     std::get<3>(k), (long long)std::get<4>(k), (long long)std::get<5>(k), kv.second.tpr,
-                     kv.second.tpb, kv.second.tile && std::get<2>(k) == kShapeSmooth ? -1 : kv.second.grid);
+    for (int keep = 0; keep < 2; keep++) {   // entries from before the tiled sweep under the header they came with
+        bool head = false;
+        for (const auto &kv : g_cache) {
+            const Key &k = kv.first;
+            const LaunchShape &sh = kv.second;
+            if ((int)sh.keep_tile != keep) continue;
+            if (!head) std::fprintf(f, "# device fp64 kind lanes rows nnz threads_per_row threads_per_block %s\n",
+                                    keep ? kHeadNoTiles : "[sweep_grid, -1: tiled sweep]");
+            head = true;
+            std::fprintf(f, "%s %d %d %d %lld %lld %d %d %d\n", std::get<0>(k).c_str(), std::get<1>(k), std::get<2>(k),
+                         std::get<3>(k), (long long)std::get<4>(k), (long long)std::get<5>(k), sh.tpr, sh.tpb,
+                         sh.tile && !keep && std::get<2>(k) == kShapeSmooth ? -1 : sh.grid);
+        }
     }
     return std::fclose(f) == 0 ? 0 : 1;
 }
@@ -222,8 +236,10 @@ int tune_cache_load(const char *path) {
     if (!f) return 1;
     char line[512], name[256];
     int bad = 0;
+    bool no_tiles = false;
     std::lock_guard<std::mutex> lk(g_mu);
     while (std::fgets(line, sizeof line, f)) {
+        if (line[0] == '#' && std::strstr(line, "[sweep_grid")) no_tiles = std::strstr(line, kHeadNoTiles) != nullptr;
         if (line[0] == '#' || line[0] == '\n') continue;
         int fp64, kind, R, tpr, tpb, grid = 0;
         long long n, nnz;
@@ -240,6 +256,7 @@ int tune_cache_load(const char *path) {
         sh.tpb = tpb;
         sh.grid = tpb == kSweepShapeTpb && grid > 0 ? grid : 0;
         sh.tile = grid == -1;   // (a level without a plan runs the colour launches of the shape)
+        sh.keep_tile = (got == 8 || no_tiles) && kind == kShapeSmooth;
         g_cache[Key{std::string(name), fp64, kind, R, (int64_t)n, (int64_t)nnz}] = sh;
     }
     std::fclose(f);
