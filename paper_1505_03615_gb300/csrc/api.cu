@@ -248,7 +248,7 @@ template <> struct P<double> {
 };
 
 // whether the level's sweeps run in the tiled kernel: it has a plan, no other launch shape was chosen, and
-// its tiles are resident at once
+// shared memory holds the blocks that its tiles want per SM
 template <class T>
 bool tiled(const Ctx &c, const DevLevel &L, int R) {
     const bool f64 = sizeof(T) == 8;
@@ -383,13 +383,8 @@ void enqueue_vcycle(Ctx &c, int R, cudaStream_t s, bool timed, Chain *ch, int to
         DevLevel &L = c.lev[d];
         if (tile(d)) {
             TileVec<T> &v = vec[d];
-            // on large levels a pass of its own: the rims would read 1.5 times the parents
-            if (L.ns > kTileProlong) {
-                launch_prolong_add<T>(L, P<T>::x(c.lev[d - 1]), v.cur ? v.y : v.x, R, s, ch);
-            } else {
-                v.xc = P<T>::x(c.lev[d - 1]);
-                v.prolong = (1u << L.tparts) - 1u;
-            }
+            v.xc = P<T>::x(c.lev[d - 1]);
+            v.prolong = (1u << L.tparts) - 1u;
             if (timed && d == top) record(c.ev_smooth[2], s, ch);
             for (int q = 0; q < c.nu2; q++)
                 launch_tile_sweep<T>(c, L, false, v, P<T>::b(L), (T *)nullptr, R, s, ch);

@@ -80,7 +80,9 @@ struct TileDev {
     int ntile = 0, nsteps = 0, maxloc = 0, maxcomp = 0, maxgrp = 0, maxquads = 0;
     int64_t groups = 0, quads = 0;
     int ring[2][3] = {{0}};                // [FP64][R = 1, 2, 4] groups in flight per warp
-    bool at_once[2][3] = {{false}};        // whether all tiles are resident at once
+    // whether shared memory holds the tiles' share of an SM, up to three blocks (registers allow three in FP32,
+    // two in FP64; the rest of the tiles then follow, no block waits for another)
+    bool at_once[2][3] = {{false}};
     int *info = nullptr, *loc = nullptr, *cum = nullptr, *map = nullptr, *row = nullptr, *qgroup = nullptr;
     int64_t *gquad = nullptr;              // [groups] quads before each group
     unsigned char *s32 = nullptr, *s64 = nullptr;

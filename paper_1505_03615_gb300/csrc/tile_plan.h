@@ -7,17 +7,16 @@
 
 namespace lbmg {
 
-constexpr int kTileSteps = 16;       // colour steps of one launch at most
-constexpr int kTileParts = 4;        // launches per sweep at most
-constexpr int kTileInfo = 24;        // ints per tile in TilePlan::info
+constexpr int kTileSteps = 8;        // colour steps of one launch at most
+constexpr int kTileParts = 2;        // launches per sweep at most
+constexpr int kTileInfo = 16;        // ints per tile in TilePlan::info
 constexpr uint16_t kTileNoRow = 0xffff;
 constexpr int kTileMinRows = 64;     // rows of a tile on small levels
 constexpr int kTileOneRound = 256;   // up to this many rows a tile, one tile per SM; then two, of
-constexpr int kTileMaxRows = 800;    // at most this many (with its rim: shared memory)
+constexpr int kTileMaxRows = 800;    // at most this many (with its rim: shared memory; 263 on 152 SMs)
 constexpr int kTileTwoParts = 12000; // from this many rows on a sweep takes two launches
 constexpr int kTileLevel32 = 80000;  // largest levels whose sweeps are tiled, FP32 and FP64
 constexpr int kTileLevel64 = 60000;
-constexpr int kTileProlong = 100000; // up to this many rows a sweep up prolongs the correction itself
 
 // Entries are stored group by group (kTileRows rows of one step, four lanes each): entry k of row l of a
 // group at 32 (base + k / 4) + 4 l + k % 4, base the quads of all groups before it, so that lane 4 l + k % 4
