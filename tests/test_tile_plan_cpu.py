@@ -48,3 +48,8 @@ def test_a_failed_host_allocation_comes_back_as_an_exception(program, tmp_path):
     """Also one that a thread of a parallel region meets: an exception that leaves the region, or a task,
     ends the process."""
     _run(program, "alloc", "sphere", tmp_path)
+
+
+@pytest.mark.parametrize("name", ["sphere", "sheet", "batch"])
+def test_every_tile_gives_the_whole_sweep_bit_for_bit(program, tmp_path, name):
+    _run(program, "plan", name, tmp_path)
