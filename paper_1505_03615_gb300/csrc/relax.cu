@@ -599,10 +599,11 @@ __global__ void __launch_bounds__(256) norm_partial_kernel(const double *__restr
     if (threadIdx.x < R) part[blockIdx.x * 4 + threadIdx.x] = t;
 }
 
-// The same for a vector of FP32 pairs: (hi + lo)^2 = hi^2 + (2 hi + lo) lo, hi^2 in FP64 and the rest, at most 2^-23
-// of it, in FP32 sums, scaled by 2^64 against underflow.  The FP64 pipe's instructions are the time (6 us each for
+// The same for a vector of FP32 pairs: (hi + lo)^2 = hi^2 + (2 hi + lo) lo, hi^2 in FP64 and the rest, mostly below
+// 2^-23 of it, in FP32 sums, scaled by 2^64 against underflow.  The FP64 pipe's instructions are the time (6 us each for
 // 927k rows of four components; all in FP64, four of them, it took 32.5 us), so hi is widened by moving its bits.
-// Numbers for which the FP32 range might not hold (below 2^-85 or from 2^30 on, but for zero) take the FP64 way.
+// Pairs for which the FP32 range might not hold (hi below 2^-85 or from 2^20 on, but for zero; lo above hi, as
+// cancellation at rounding level can leave it) take the FP64 way.
 constexpr float kPairScale = 1.8446744073709552e19f;   // 2^64
 
 __device__ __forceinline__ double pair_sum(float hi, float lo) {   // (volatile: not before its branch is taken)
@@ -644,8 +645,8 @@ __global__ void __launch_bounds__(256) norm_pair_partial_kernel(const float *__r
         for (int u = 0; u < U; u++)
 #pragma unroll
             for (int r = 0; r < R; r++) {
-                const unsigned a = __float_as_uint(h[u][r]) & 0x7fffffffu;   // |hi|
-                usual = usual && (a - 0x15000000u < 0x39800000u || (a == 0u && l[u][r] == 0.f));
+                const unsigned a = __float_as_uint(h[u][r]) & 0x7fffffffu, al = __float_as_uint(l[u][r]) & 0x7fffffffu;
+                usual = usual && (a - 0x15000000u < 0x34800000u || a == 0u) && al <= a;
             }
         if (usual) {
 #pragma unroll
