@@ -240,7 +240,9 @@ int lbmg_project_rhs(lbmg_handle h, const double *f_vertex, int nrhs, double *rh
  * level on the way down, residual, restriction P^T r, the coarsest solve, then
  * prolongation x += P e and ν2 sweeps on the way up (Section 4.3).  precision:
  * LBMG_FP64 runs the whole cycle in FP64; LBMG_MIXED runs it in FP32 inside an
- * FP64 defect-correction loop (residual and update in FP64).  Stops when
+ * FP64 defect-correction loop (residual and update in FP64, with the values
+ * carried as FP32 pairs and rhs as three FP32 numbers on levels with a packed
+ * copy: as accurate as lbmg_residual_split, within FP32's range).  Stops when
  * ||rhs - A x||_2 <= tol ||rhs||_2 for every right-hand side (||rhs - A x||_2 <=
  * tol when rhs = 0), or after max_cycles.  x: [n_depth][nrhs], in/out (warm
  * start).  stats may be NULL.
@@ -318,10 +320,11 @@ int lbmg_cmcf_step(lbmg_handle h, const double *X, double delta, double *x, doub
 int lbmg_eigs(lbmg_handle h, int k, double tol, int max_iters, const double *X0, double *lambda, double *X,
               double *residuals, int *iters, void *stream);
 
-/* Number of kernels each call launches: lbmg_assemble, lbmg_project_rhs, one
-   V-cycle step of lbmg_solve/lbmg_vcycles in `precision` (cycle + FP64 residual
-   + norms; 0 for the persistent solve, whose cycles run inside its one launch),
-   and the fixed part of lbmg_solve around its cycles.  Host only. */
+/* Number of kernels each call launches: lbmg_assemble (after the first, which has the
+   build-time geometry's besides), lbmg_project_rhs, one step of lbmg_solve/lbmg_vcycles in
+   `precision` with four right-hand sides (cycle + FP64 residual + norms, without the graph's
+   stopping test; 0 for the persistent solve, whose cycles run inside its one launch), and
+   the fixed part of lbmg_solve around its cycles.  Nothing runs on the device. */
 int lbmg_launch_counts(lbmg_handle h, int precision, int *assemble, int *project_rhs, int *per_cycle,
                        int *solve_fixed);
 
@@ -388,7 +391,8 @@ int lbmg_residual(lbmg_handle h, int d, const double *rhs, const double *x, doub
    lbmg_residual computes it, arguments and layout the same, with FP64 values carried as
    pairs of FP32 numbers (value = hi + lo): every product a x = ah xh + (ah xl + al xh + the
    exact rounding error of ah xh) and every partial sum is an FP32 pair (Knuth's two-sum),
-   and rhs - sum is formed in FP64.  The result agrees with the FP64 residual to about 2^-44
+   and rhs - sum is formed in FP64 (the solve forms it from three FP32 parts of rhs, to the same
+   accuracy).  The result agrees with the FP64 residual to about 2^-44
    of sum_j |a_ij x_j| (the dropped al xl term and FP32 rounding of the small terms).  Why:
    GB300 executes FP64 arithmetic at a small fraction of its FP32 rate, which made the FP64
    residual of the finest level compute-bound.  Levels with a packed copy only (not the

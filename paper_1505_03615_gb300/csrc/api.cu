@@ -1946,53 +1946,50 @@ int lbmg_prolong_add(lbmg_handle h, int d, const double *x_coarse, double *x_fin
     return finish_output(x_fine, out, (size_t)Lf.n * nrhs, host_out, s);
 }
 
+// kernels of one iteration of the V-cycle solve, counted in a capture of it (nothing runs)
+static int count_iteration(Ctx &c, int precision, int *kernels) {
+    cudaStream_t s = c.capture_stream;
+    LBMG_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    enqueue_iteration(c, 4, precision, s);
+    cudaGraph_t graph = nullptr;
+    LBMG_CK(cudaStreamEndCapture(s, &graph));
+    size_t n = 0;
+    cudaError_t e = cudaGraphGetNodes(graph, nullptr, &n);
+    std::vector<cudaGraphNode_t> nodes(n);
+    if (e == cudaSuccess) e = cudaGraphGetNodes(graph, nodes.data(), &n);
+    *kernels = 0;
+    for (size_t q = 0; q < n && e == cudaSuccess; q++) {
+        cudaGraphNodeType type;
+        e = cudaGraphNodeGetType(nodes[q], &type);
+        if (e == cudaSuccess && type == cudaGraphNodeTypeKernel) (*kernels)++;
+    }
+    cudaGraphDestroy(graph);
+    LBMG_CK(e);
+    return LBMG_OK;
+}
+
 int lbmg_launch_counts(lbmg_handle h, int precision, int *assemble, int *project_rhs, int *per_cycle,
                        int *solve_fixed) {
     if (!h) return LBMG_INVALID_ARG;
-    const Ctx &c = h->c;
-    const int levels = c.D - c.d0;
-    if (assemble) *assemble = 2 + levels + (levels + 1) + 3;
-    if (project_rhs) *project_rhs = 2;
-    auto per_sweep = [&](const int *cs) {
-        if (c.smoother == LBMG_JACOBI) return 2;
-        int k = 0;
-        for (int q = 0; q < 8; q++) k += cs[q + 1] > cs[q];
-        return k;
-    };
-    int cyc = 0;
-    if (c.gamma == 1 && !c.coarse_smooth) {
-        const bool narrow = one_block<float>(c, c.persist_dn, 4) && c.smoother != LBMG_JACOBI && precision == LBMG_MIXED;
-        const bool smem = c.narrow.dn >= c.d0 && c.smoother != LBMG_JACOBI && precision == LBMG_MIXED;
-        const int bottom = smem ? c.narrow.dn : (narrow ? c.persist_dn : c.d0);
-        cyc = 1;   // the one-block bottom cycle, or the coarse apply
-        for (int d = bottom + 1; d <= c.D; d++) {   // sweeps, residual, restriction, prolongation
+    Ctx &c = h->c;
+    if (assemble) {   // the finest entries and a product, two for the diagonals, packed copy and tiles per level, factor
+        int k = 1 + 3 * (c.D - c.d0) + 2 + (c.ncblk > 0 ? 3 : 0);
+        for (int d = c.d0 + 1; d <= c.D; d++) {
             const DevLevel &L = c.lev[d];
-            if (c.nu1 > 0 && c.nu2 > 0 && c.smoother != LBMG_JACOBI && L.tparts > 0 &&
-                L.tonce[precision == LBMG_FP64][2] && L.shape[precision == LBMG_FP64][kShapeSmooth].tile) {   // sweeps, residual, restriction
-                cyc += (c.nu1 + c.nu2) * L.tparts + (L.tfused ? 0 : 1) + 1 + (L.ncb > 0);
-                continue;
-            }
-            const bool whole = precision == LBMG_MIXED && c.smoother != LBMG_JACOBI &&
-                               L.shape[0][kShapeSmooth].tpb == kSweepShapeTpb && L.pk_map && c.sweep_bar;
-            if (whole) cyc += (c.nu1 > 0) + (c.nu2 > 0);   // one cooperative launch per smoothing
-            else {
-                cyc += (c.nu1 + c.nu2) * per_sweep(L.cs);
-                // below the finest level the restriction does colour 0 of the first sweep
-                if (d < c.D && c.smoother != LBMG_JACOBI && c.nu1 > 0 && L.cs[1] > L.cs[0]) cyc -= 1;
-            }
-            cyc += 3 + (L.ncb > 0);
+            k += (L.pk_map != nullptr) + 2 * L.tparts + (L.tparts > 0 && !L.tfused);
         }
-    } else {
-        // the general cycle: gamma visits of each coarser level
-        long visit = c.coarse_smooth ? (long)(c.nu1 + c.nu2) * per_sweep(c.lev[c.d0].cs_all) : 1;
-        for (int d = c.d0 + 1; d <= c.D; d++) visit = (long)(c.nu1 + c.nu2) * per_sweep(c.lev[d].cs) + 3 + c.gamma * visit;
-        cyc = (int)std::min<long>(visit, 1 << 30);
+        *assemble = k;
     }
-    cyc += (precision == LBMG_MIXED ? 2 : 1) + 1 + 2;   // conversion/update, FP64 residual, norms
-    const bool persistent = c.persistent && c.persist_ok && c.smoother == LBMG_GS_COLOURED;
+    if (project_rhs) *project_rhs = 2;
     // the persistent solve runs every cycle inside one launch: two packs, the solve, one unpack
-    if (per_cycle) *per_cycle = persistent ? 0 : cyc;
-    if (solve_fixed) *solve_fixed = persistent ? 4 : 2 + 1 + 2 + 2 + 1;
+    const bool persistent = c.persistent && c.persist_ok && c.smoother == LBMG_GS_COLOURED;
+    if (per_cycle) {
+        *per_cycle = 0;
+        if (!persistent) LBMG_TRY(count_iteration(c, precision, per_cycle));
+    }
+    // packs, residual, norms of b and r, unpack; the iterate's and right-hand side's parts there and back
+    const bool pairs = pair_iterate(c, precision, false);
+    if (solve_fixed) *solve_fixed = persistent ? 4 : 2 + 1 + 2 + 2 + 1 + (pairs ? (c.learned_on ? 3 : 4) : 0);
     return LBMG_OK;
 }
 
