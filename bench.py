@@ -828,7 +828,9 @@ def main():
         tpr, tpb = shapes[str(D)][0]
         kname = "pk_row_kernel" if tpr == 4 else "smooth_colour_kernel"
         kernel = f"{kname}<float,{R},GS> (finest level, one colour, {tpr} threads per row, {tpb} threads/block)"
-        if (tpr, tpb) == (4, 256) and n <= 80_000:   # the default shape stands for the tiled sweep there
+        # a tiled level reports the default shape; setting one by hand turns its tiles off (all timing is done)
+        L.lbmg_set_launch_shape(h, D, L.LBMG_MIXED, 0, tpr, tpb)
+        if L.lbmg_launch_counts(h, L.LBMG_MIXED)[2] != per_cycle:
             kernel = f"tile_kernel<float,{R}> (finest level; an eighth of a sweep, transfers of its launches included)"
         key = f"{kname}_gs_{workload}"
     achieved = launch_bytes / (avg_launch_ms * 1e-3) / 1e9 if avg_launch_ms > 0 else 0.0
@@ -867,16 +869,17 @@ def main():
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "f32 relax / f64 assembly, residual with f64 values as f32 pairs", "data": "synthetic",
+            "dtype": "f32 relax / f64 assembly, residual with f64 values as f32 pairs (right-hand side as three f32), norms in f64", "data": "synthetic",
             "config": {"workload": workload, "triangles": int(F.shape[0]), "depth": depth, "min_depth": d0,
                        "dofs_finest": n, "nnz_finest": nnz, "fragments_finest": nfrag, "nrhs": nrhs, "t": t,
                        "tol": tol, "precision": "mixed", "l2": "inputs larger than L2 (assembly streams >0.5 GB/step)",
                        "cycle": f"{args.cycle.upper()}({args.nu},{args.nu})",
                        "assembly": ("every step: the finest entries gathered from the pieces' local integrals (mass "
                                     "scaled by the current area weights), the Galerkin products of every coarser "
-                                    "level, A = M + tL and its packed and FP32 copies; the pieces' moments and local "
-                                    "integrals depend only on the build-time geometry and are computed by the first "
-                                    "assembly (setup)"),
+                                    "level, A = M + tL and its packed, tiled and FP32 copies; the pieces' moments and "
+                                    "local integrals and the stiffness of every level depend only on the build-time "
+                                    "geometry and are computed by the first assembly (setup): later ones sum the mass "
+                                    "and read the stiffness"),
                        "parallelism": "replicas" if ws > 1 else "single",
                        "solve": ("persistent (one cooperative launch)" if args.persistent else
                                  "one graph launch per solve (conditional loop, device stopping test)"),

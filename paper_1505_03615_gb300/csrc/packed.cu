@@ -76,9 +76,10 @@ __device__ __forceinline__ void load_row<double, 4>(const double *p, double (&v)
 // still zero and are left out without a look at x, so that x need not be zeroed and half the gathers fall
 // away.
 // NC of the R components are live (three right-hand sides padded to four); each is summed, updated and written
-// by a lane of its own.  GB300's FP64 pipe takes a warp instruction in 64 cycles or so, and the FP64 kernels are
-// bound by their number: eight rows of 18 entries take 20 for three right-hand sides, where four components
-// summed by every lane and updated by one took 36 (an FP64 sweep of 927k rows: 388 -> 250 us).
+// by a lane of its own.  An SM's FP64 pipe takes a warp instruction in 16 cycles, and the FP64 kernels are bound by
+// their number (pipe 77% active): 29 per eight rows for three right-hand sides, 3 for each of the eight quads below
+// whether the rows have it or not, and 5 for the sums and the update; four components summed by every lane and
+// updated by one took more (an FP64 sweep of 927k rows: 361 -> 232 us).
 // One warp per group.  kGs: Gauss-Seidel update x += (b - A x) / A_ii (rows of one
 // colour, which never couple); otherwise r = b - A x.  Before the grid-dependency wait
 // a warp loads its group, its entries and (kGs) the inverse diagonal; after it, the
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(256) pk_split_residual_kernel(int g1, const in
 // right-hand side (z, when given, zeroed as its start), and what the rounding left (rlo), which the norms need:
 // of r rounded alone they were off by up to 1e-8 of themselves on some hundred rows.  The right-hand side comes
 // as three FP32 numbers (53 bits, down to FP32's smallest numbers, where the products' pairs end too) and is
-// subtracted as pairs, so that no FP64 instruction is left (a warp issues one in about 64 cycles).  The norms
+// subtracted as pairs, so that no FP64 instruction is left (an SM takes one in 16 cycles).  The norms
 // are a pass of their own over r32 and rlo: summed here, the FP64 additions at every block's end held its place
 // (94 -> 140 us).  NC of the R components are live.
 template <int R, int NC>

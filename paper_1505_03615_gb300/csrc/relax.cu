@@ -113,7 +113,7 @@ __device__ __forceinline__ void group_sum(T (&acc)[R]) {
 }
 
 // sums of the components over a warp, halved across its lanes so that an FP64 sum takes 6 additions of 4
-// components instead of 20 (GB300's FP64 pipe takes 64 cycles a warp instruction): one lane per component
+// components instead of 20 (an SM's FP64 pipe takes a warp instruction in 16 cycles): one lane per component
 // returns its sum and the component in comp, the others -1
 template <class T, int R>
 __device__ __forceinline__ T warp_sum(const T (&a)[R], int lane, int &comp) {

@@ -15,10 +15,14 @@
 // 64 rows a tile, 1.5 to 2 at 250 rows in two launches per sweep of four colours each, and every plan has a
 // copy of the entries, which on larger levels pushes the other levels' data out of L2.  Measured per FP32
 // sweep of torus-knot levels, colour launches / tiles: 18 / 5.5 us at 5,000 rows, 18 / 7.5 at 19,000, 18 / 11
-// at 78,000, 28 / 27 at 232,000, 76 / 71-79 at 927,000; a cycle of the 1M-triangle sheets with four
-// components took 1410 us with 91,000 rows tiled, 1283 without.  FP64 at three right-hand sides: 42 / 14 us,
-// 42 / 30, 42 / 37, 60 / 70, 290 / 310, with colour launches that summed the padding lane too; without it the
-// line still holds (a cycle of the 200k knot 608 us with it at 60,000 rows, 632 with it at 15,000).
+// at 78,000, 28 / 27 at 232,000, 76 / 71-79 at 927,000.  It depends on the components and on what else has to
+// stay in L2: a cycle of the 1M-triangle sheets with their 91,202 rows tiled / not took 852 / 860 us at one
+// right-hand side, 1007 / 1011 at two, 1246 / 1239 at three, with the next level of 359,326 rows tiled too
+// 895, 1068 and 1244; between 77,584 and 91,202 rows nothing was measured, and 80,000 is a coarse line.  FP64 at
+// three right-hand sides: 42 / 14 us, 42 / 30, 42 / 37, 60 / 70, 290 / 310, with colour launches that summed the
+// padding lane too; without it the line still holds (a cycle of the 200k knot 608 us with it at 60,000 rows, 632
+// with it at 15,000).  Plans for FP64 exist up to kTileLevel32: the tuner takes them at 77,584 rows for one and
+// two right-hand sides.
 //
 // Four lanes share a row, as in packed.cu, so that a row's gathers are few per lane and all in flight
 // together (a step is one chain of shared-memory latencies); the lanes' sums are added so that lane c ends
