@@ -556,7 +556,7 @@ static void launch_tile(const DevLevel &L, const TileDev &t, int part, const Til
     a.xout = ((v.cur >> part) & 1u) ? v.x : v.y;
     a.xc = v.xc; a.par = L.par; a.npl2 = L.npl2; a.r = r;
     a.status = c.narrow.status;
-    a.arrivals = kTileWarps + c.barrier_phantoms;
+    a.arrivals = kTileWarps + std::min(c.barrier_phantoms, 1024);   // (a barrier counts to 2^20)
     a.wait_ns = c.barrier_phantoms > 0 ? kTilePhantomWaitNs : kTileWaitNs;
     auto k = R == 1 ? tile_kernel<T, 1, 1> : R == 2 ? tile_kernel<T, 2, 2>
              : c.lanes == 3 ? tile_kernel<T, 4, 3> : tile_kernel<T, 4, 4>;
